@@ -1448,46 +1448,66 @@ k_apply_combine2(const double* __restrict__ sums, int nf, const d4* __restrict__
     }
 }
 
-// per face: z = (r/a) W_S - (H W)_S in FP64, then the corner values of the
-// transposed map: 2 a_S grad phi_c . zV (B) and 2 a_S zU / 3 (B0, L)
-// (perm != null: the partials are in sorted order, thread t combines face
-// perm[t] from partial row t)
+// z = (r/a) W_S - (H W)_S in FP64 per (face, column), then the corner values of
+// the transposed map: 2 a_S grad phi_c . zV (B) and 2 a_S zU / 3 (B0, L)
+// (perm != null: the partials are in sorted order, position t combines face
+// perm[t] from partial row t). A block takes 32 positions x (KC columns + the
+// areas), one thread each: the lanes of a warp read consecutive positions of one
+// partial row, and a thread's sums advance together over the splits, four at a
+// time, so that up to 16 loads are in flight. Bound by the FP64 pipe on large
+// meshes (17 operations per thread) and by latency on small ones.
 template <int OP, int KC>
-__global__ void k_apply_combine(const double* __restrict__ part, int nsplit, int nf,
-                                const d4* __restrict__ f64a, const double* __restrict__ fgrad,
-                                const double* __restrict__ W64, int k, int col0,
-                                double* __restrict__ corner, const int* __restrict__ perm) {
+__global__ void __launch_bounds__(32 * (KC + 1))
+k_apply_combine(const double* __restrict__ part, int nsplit, int nf, const d4* __restrict__ f64a,
+                const double* __restrict__ fgrad, const double* __restrict__ W64, int k, int col0,
+                double* __restrict__ corner, const int* __restrict__ perm) {
     using L = OpLayout<OP, KC>;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nf) return;
-    const int S = perm ? perm[t] : t;
-    double s[L::NA];
-    for (int i = 0; i < L::NA; ++i) {
-        double x = 0.0;
-        for (int sp = 0; sp < nsplit; ++sp) x += part[((size_t)sp * L::NA + i) * nf + t];
-        s[i] = x;
-    }
-    double a = f64a[S].w;
-    const double* W = W64 + 4 * KC * (size_t)S;
-    double zV[3 * KC], zU[KC];
-    for (int i = 0; i < 3 * KC; ++i) zV[i] = 0.0;
-    for (int i = 0; i < KC; ++i) zU[i] = 0.0;
-    int o = 0;
-    if (L::HIGH) {
-        double r = s[0] / a;
-        for (int i = 0; i < 3 * KC; ++i) zV[i] = r * W[i] - s[1 + i];
-        o = 1 + 3 * KC;
-    }
-    if (L::USEU) {
-        double r = s[o] / a;
-        for (int c = 0; c < KC; ++c) zU[c] = r * W[3 * KC + c] - s[o + 1 + c];
-    }
-    for (int cr = 0; cr < 3; ++cr)
-        for (int c = 0; c < KC && col0 + c < k; ++c) {
-            double g = 0.0;
-            for (int q = 0; q < 3; ++q) g += fgrad[9 * S + 3 * cr + q] * zV[q * KC + c];
-            corner[((size_t)S * 3 + cr) * k + col0 + c] = 2.0 * a * (g + zU[c] * (1.0 / 3.0));
+    __shared__ double s_hi[32], s_lo[32];
+    const int fl = threadIdx.x, c = threadIdx.y;
+    const int t = blockIdx.x * 32 + fl;
+    const bool has = t < nf;
+    const int S = has ? (perm ? perm[t] : t) : 0;
+    const double a = has ? f64a[S].w : 1.0;
+    double hV[3] = {0.0, 0.0, 0.0}, hU = 0.0;
+    const bool mine = has && c < KC && col0 + c < k;
+    if (has && c == KC) {   // the areas' sums
+        const double ia = 1.0 / a;
+        double hi = 0.0, lo = 0.0;
+#pragma unroll 4
+        for (int sp = 0; sp < nsplit; ++sp) {
+            const double* ps = part + (size_t)sp * L::NA * nf + t;
+            if (L::HIGH) hi += ps[0];
+            if (L::USEU) lo += ps[(size_t)L::NH * nf];
         }
+        s_hi[fl] = hi * ia;
+        s_lo[fl] = lo * ia;
+    } else if (mine) {
+#pragma unroll 4
+        for (int sp = 0; sp < nsplit; ++sp) {
+            const double* ps = part + (size_t)sp * L::NA * nf + t;
+            if (L::HIGH) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) hV[q] += ps[(size_t)(1 + q * KC + c) * nf];
+            }
+            if (L::USEU) hU += ps[(size_t)(L::NH + 1 + c) * nf];
+        }
+    }
+    __syncthreads();
+    if (!mine) return;
+    const double* W = W64 + 4 * KC * (size_t)S;
+    double zV[3], zU = 0.0;
+    if (L::HIGH)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) zV[q] = s_hi[fl] * W[q * KC + c] - hV[q];
+    if (L::USEU) zU = (s_lo[fl] * W[3 * KC + c] - hU) * (1.0 / 3.0);
+    const double* gr = fgrad + 9 * (size_t)S;
+    const double a2 = 2.0 * a;
+#pragma unroll
+    for (int cr = 0; cr < 3; ++cr) {
+        double g = zU;
+        if (L::HIGH) g += gr[3 * cr] * zV[0] + gr[3 * cr + 1] * zV[1] + gr[3 * cr + 2] * zV[2];
+        corner[((size_t)S * 3 + cr) * k + col0 + c] = a2 * g;
+    }
 }
 
 template <typename T, int OP, int KC>
@@ -1524,7 +1544,7 @@ static int launch_apply_op(tp_mesh* m, const tp_params* p, const double* v, int 
                                                         g.tiles_per_split, T(s), T(l_exp), m->part.as<double>());
         }
         TP_LAUNCH_CHECK();
-        k_apply_combine<OP, KC><<<(nf + 255) / 256, 256, 0, st>>>(m->part.as<double>(), g.nsplit, nf,
+        k_apply_combine<OP, KC><<<(nf + 31) / 32, dim3(32, KC + 1), 0, st>>>(m->part.as<double>(), g.nsplit, nf,
                                                                   m->f64a.as<d4>(), m->fgrad.as<double>(),
                                                                   m->wv64.as<double>(), k, col0,
                                                                   m->corner.as<double>(), nullptr);
@@ -2567,7 +2587,7 @@ static int launch_bh_apply_op(tp_mesh* m, const tp_params* p, const double* v, i
                     (float)(p->theta * p->theta), (float)s, (float)l_exp, m->part.as<double>(), cnt);
         }
         TP_LAUNCH_CHECK();
-        k_apply_combine<OP, KC><<<(nf + 255) / 256, 256, 0, st>>>(m->part.as<double>(), 1, nf,
+        k_apply_combine<OP, KC><<<(nf + 31) / 32, dim3(32, KC + 1), 0, st>>>(m->part.as<double>(), 1, nf,
                                                                   m->f64a.as<d4>(), m->fgrad.as<double>(),
                                                                   m->wv64.as<double>(), k, col0,
                                                                   m->corner.as<double>(), bv.perm);
