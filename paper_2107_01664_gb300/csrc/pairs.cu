@@ -39,7 +39,15 @@ __device__ __forceinline__ float rcp_(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ double rcp_(double x) { return 1.0 / x; }
+// FP64 reciprocal: the 20-bit approximation and one third-order step, three
+// FP64 operations in place of the division's sequence (the FP64 pipe issues
+// two lanes a cycle and SM and bounds every FP64 kernel); error below one ulp
+__device__ __forceinline__ double rcp_(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return __double2hiint(x) == 0x7ff00000 ? 0.0 : fma(y, fma(e, e, e), y);
+}
 
 __device__ __forceinline__ float lg2_(float x) {
     float r;
@@ -54,6 +62,59 @@ __device__ __forceinline__ float ex2_(float x) {
 // x^y for x >= 0 (x = 0 gives 0 for y > 0)
 __device__ __forceinline__ float pow_(float x, float y) { return ex2_(y * lg2_(x)); }
 __device__ __forceinline__ double pow_(double x, double y) { return pow(x, y); }
+
+// x^{-a} in FP64 for a rational a = k / n with a small n (n = 0: pow). With
+// u = x^{-1/n} from the FP32 MUFU (relative error about 1e-6) and e = 1 - x u^n,
+//   x^{-a} = u^k (1 - e)^{-a} = u^k (1 + a e + a (a+1)/2 e^2 + a (a+1) (a+2)/6 e^3 + ..),
+// whose next term is below 1e-18. About 12 FP64 operations at n = 3 (p = 6) in
+// place of about 100 for pow. x outside FP32's range takes pow.
+struct RootPow {
+    int n = 0, k = 0;
+    float inv = 0.f;   // -1 / n
+    double a = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0;
+};
+
+__device__ __forceinline__ double ipow_(double u, int k) {   // u^k, k >= 1
+    double r = 1.0, b = u;
+    bool first = true;
+    for (;;) {
+        if (k & 1) {
+            r = first ? b : r * b;
+            first = false;
+        }
+        k >>= 1;
+        if (!k) break;
+        b *= b;
+    }
+    return r;
+}
+
+// x^{-a}; *ix = 1/x. The conversions between FP32 and FP64 would run on the
+// FP64 pipe: normal numbers are converted by shifting the bits instead (x
+// truncated to FP32, which only moves the seed by 2^-23).
+__device__ __forceinline__ double root_pow(double x, const RootPow& rp, double* ix) {
+    const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
+    // 2^-100 <= x < 2^100
+    if (rp.n == 0 || xh - ((1023u - 100u) << 20) >= (200u << 20)) {
+        *ix = rcp_(x);
+        return pow_(x, -rp.a);
+    }
+    const float xf = __uint_as_float(__funnelshift_l(xl, xh, 3) - ((1023u - 127u) << 23));
+    const unsigned uf = __float_as_uint(ex2_(lg2_(xf) * rp.inv));
+    const double u = __hiloint2double((int)((uf >> 3) + ((1023u - 127u) << 20)), (int)(uf << 29));
+    double un, uk;
+    if (rp.n == 3) {
+        const double u2 = u * u, u4 = u2 * u2;
+        un = u2 * u;
+        uk = rp.k == 5 ? u4 * u : rp.k == 4 ? u4 : ipow_(u, rp.k);
+    } else {
+        un = ipow_(u, rp.n);
+        uk = ipow_(u, rp.k);
+    }
+    const double e = fma(-x, un, 1.0);
+    *ix = fma(un, fma(e, fma(e, e, e), e), un);
+    return fma(uk * e, fma(fma(rp.c3, e, rp.c2), e, rp.c1), uk);
+}
 
 // smallest |d|^2 treated as a real pair; the self pair has d = 0 exactly
 template <typename T> __device__ __forceinline__ T tiny_r2();
@@ -280,6 +341,43 @@ static Grid make_grid(int nt, int nf, int tt, int per_sm) {
     return g;
 }
 
+// FP64 kernels run at the rate of an SM's FP64 pipe however many blocks it
+// holds, so what counts is that every SM gets the same number of tiles. Hence at
+// least eight blocks per SM, where there are tiles for it, and two resident (the
+// second hides the tile loads; a third can only take blocks of the last wave from
+// an SM with none). 3,000 faces, A on 3 columns: FP64 pipe busy 83% of the launch
+// and 92% of the SMs' active time; 0.76 ms, 2.29 ms with pow and two-tile blocks.
+static Grid fp64_grid(Grid g, int nf) {
+    const int ntiles = (nf + NT - 1) / NT;
+    const int want = std::min(ntiles, (8 * sm_count() + g.bx - 1) / g.bx);
+    if (g.nsplit >= want) return g;
+    g.tiles_per_split = std::max(1, ntiles / want);
+    g.nsplit = (ntiles + g.tiles_per_split - 1) / g.tiles_per_split;
+    return g;
+}
+
+// dynamic shared memory that leaves room for two blocks of a kernel per SM
+template <class F>
+static size_t two_resident(F* fn) {
+    int dev = 0, sm = 0, reserved = 0;
+    cudaFuncAttributes at{};
+    cudaGetDevice(&dev);
+    if (cudaFuncGetAttributes(&at, (const void*)fn) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    // more than a third of the SM's memory per block, at most a half
+    const long want = (long)sm / 2 - reserved - (long)at.sharedSizeBytes - 4096;
+    if (want <= 0) return 0;
+    if (cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return (size_t)want;
+}
+
 // ===========================================================================
 // energy rows, Eq. 10: sum_{T != S} K(S,T) a_T  (times a_S in the combine)
 // ===========================================================================
@@ -440,6 +538,7 @@ static int launch_energy(tp_mesh* m, const tp_params* p, const int32_t* tl, int 
     using V4 = typename V4T<T>::type;
     constexpr int TT = sizeof(T) == 4 ? 4 : 2;
     Grid g = make_grid(nt, m->nf, TT, resident_per_sm((const void*)k_energy<T, true, TT>, NT));
+    if (sizeof(T) == 8) g = fp64_grid(g, m->nf);
     TP_TRY(ensure(m->part, sizeof(double) * (size_t)g.nsplit * nt));
     const V4* fa = (const V4*)(sizeof(T) == 4 ? m->f32a.ptr : m->f64a.ptr);
     const V4* fb = (const V4*)(sizeof(T) == 4 ? m->f32b.ptr : m->f64b.ptr);
@@ -449,11 +548,11 @@ static int launch_energy(tp_mesh* m, const tp_params* p, const int32_t* tl, int 
     {
         ProfScope ps(m, PK_ENERGY, units, st);
         if (p->p == 6.0)
-            k_energy<T, true, TT><<<grid, NT, 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
+            k_energy<T, true, TT><<<grid, NT, sizeof(T) == 8 ? two_resident(k_energy<T, true, TT>) : 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
                                                        m->center.as<double>(), m->nf, tl, nt,
                                                        g.tiles_per_split, T(3), m->part.as<double>());
         else
-            k_energy<T, false, TT><<<grid, NT, 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
+            k_energy<T, false, TT><<<grid, NT, sizeof(T) == 8 ? two_resident(k_energy<T, false, TT>) : 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
                                                         m->center.as<double>(), m->nf, tl, nt,
                                                         g.tiles_per_split, T(0.5 * p->p), m->part.as<double>());
         TP_LAUNCH_CHECK();
@@ -686,6 +785,7 @@ static int launch_diff(tp_mesh* m, const tp_params* p, double* adj, double* erow
     using V4 = typename V4T<T>::type;
     constexpr int TT = sizeof(T) == 4 ? 2 : 1;
     Grid g = make_grid(m->nf, m->nf, TT, resident_per_sm((const void*)k_diff<T, true, TT>, NT));
+    if (sizeof(T) == 8) g = fp64_grid(g, m->nf);
     TP_TRY(ensure(m->part, sizeof(double) * (size_t)g.nsplit * NADJ * m->nf));
     const V4* fa = (const V4*)(sizeof(T) == 4 ? m->f32a.ptr : m->f64a.ptr);
     const V4* fb = (const V4*)(sizeof(T) == 4 ? m->f32b.ptr : m->f64b.ptr);
@@ -695,11 +795,11 @@ static int launch_diff(tp_mesh* m, const tp_params* p, double* adj, double* erow
     {
         ProfScope ps(m, PK_DIFF, units, st);
         if (p->p == 6.0)
-            k_diff<T, true, TT><<<grid, NT, 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
+            k_diff<T, true, TT><<<grid, NT, sizeof(T) == 8 ? two_resident(k_diff<T, true, TT>) : 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
                                                      m->center.as<double>(), m->nf, g.tiles_per_split, T(2),
                                                      m->part.as<double>());
         else
-            k_diff<T, false, TT><<<grid, NT, 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
+            k_diff<T, false, TT><<<grid, NT, sizeof(T) == 8 ? two_resident(k_diff<T, false, TT>) : 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
                                                       m->center.as<double>(), m->nf, g.tiles_per_split,
                                                       T(0.5 * p->p - 1.0), m->part.as<double>());
         TP_LAUNCH_CHECK();
@@ -810,6 +910,8 @@ __global__ void k_face_W(const double* __restrict__ v, int k, int col0, const in
     T* out = reinterpret_cast<T*>(Wp) + (size_t)S * 4 * nw4;
     const bool hi = (op == TP_OP_A || op == TP_OP_B), lo = op != TP_OP_B;
     const int ou = hi ? 1 + 3 * KC : 0;   // start of the low-order block in out
+    // the FP64 kernel leaves the factor 1/2 of the low-order kernel to X (exact)
+    const double half = sizeof(T) == 8 && (op == TP_OP_A || op == TP_OP_B0) ? 0.5 : 1.0;
     for (int c = 0; c < CG && c0 + c < KC; ++c) {
         for (int q = 0; q < 3; ++q) {
             double gq = 0.0;
@@ -820,11 +922,11 @@ __global__ void k_face_W(const double* __restrict__ v, int k, int col0, const in
         }
         const double wu = a * (val[0][c] + val[1][c] + val[2][c]) * (1.0 / 3.0);
         w64[3 * KC + c0 + c] = wu;
-        if (lo) out[ou + 1 + c0 + c] = (T)wu;
+        if (lo) out[ou + 1 + c0 + c] = (T)(half * wu);
     }
     if (g == 0) {
         if (hi) out[0] = (T)a;
-        if (lo) out[ou] = (T)a;
+        if (lo) out[ou] = (T)(half * a);
         for (int n = ou + (lo ? 1 + KC : 0); n < 4 * nw4; ++n) out[n] = T(0);
     }
 }
@@ -906,10 +1008,26 @@ __device__ __forceinline__ typename P2T<T>::type p2zero() {
 template <typename T, int OP, bool SELF, int KC>
 __device__ __forceinline__ void apply_term(T dx, T dy, T dz, T nx, T ny, T nz, T mx, T my, T mz,
                                            const typename P2T<T>::type* x2, T s_exp, T l_exp,
-                                           typename P2T<T>::type* pt) {
+                                           typename P2T<T>::type* pt, const RootPow& rp = RootPow()) {
     using L = OpLayout<OP, KC>;
     constexpr bool LOW = (OP == TP_OP_A || OP == TP_OP_B0);
     T r2 = r2_eps(dx, dy, dz);
+    if constexpr (sizeof(T) == 8) {
+        double ir2;
+        // the self pair (|d|^2 = tiny, outside root_pow's range) is taken at 1 and dropped
+        const bool own = SELF && !(r2 > T(2) * tiny_r2<T>());
+        double h = root_pow(own ? 1.0 : r2, rp, &ir2);   // |d|^{-2s}, or the kernel of L
+        if (SELF) h = own ? T(0) : h;
+#pragma unroll
+        for (int i = 0; i < (OP == TP_OP_L ? L::NA : L::NH) / 2; ++i) pt[i] = pfma(h, x2[i], pt[i]);
+        if (LOW) {
+            const double uS = nx * dx + ny * dy + nz * dz, uT = mx * dx + my * dy + mz * dz;
+            const double h0 = (fma(uS, uS, uT * uT) * (ir2 * ir2)) * h;   // its factor 1/2 is in X
+#pragma unroll
+            for (int i = L::NH / 2; i < L::NA / 2; ++i) pt[i] = pfma(h0, x2[i], pt[i]);
+        }
+        return;
+    }
     if (OP == TP_OP_L) {
         T h = pow_(r2, -l_exp);
         if (SELF) h = r2 > T(2) * tiny_r2<T>() ? h : T(0);
@@ -936,7 +1054,7 @@ __global__ void __launch_bounds__(NT)
 k_apply(const typename V4T<T>::type* __restrict__ fa, const typename V4T<T>::type* __restrict__ fb,
         const float4* __restrict__ flo, const float4* __restrict__ tbox, const double* __restrict__ center,
         const typename V4T<T>::type* __restrict__ Wp, int nf, int tiles_per_split, T s_exp,
-        T l_exp, double* __restrict__ part) {
+        T l_exp, double* __restrict__ part, RootPow rp) {
     using V4 = typename V4T<T>::type;
     using L = OpLayout<OP, KC>;
     constexpr bool LOW = (OP == TP_OP_A || OP == TP_OP_B0);
@@ -1023,7 +1141,7 @@ k_apply(const typename V4T<T>::type* __restrict__ fa, const typename V4T<T>::typ
                     for (int j = 0; j < TT; ++j)
                         apply_term<T, OP, true, KC>((tx[j] - s.x) + (T)(lx[j] - l.x), (ty[j] - s.y) + (T)(ly[j] - l.y),
                                                     (tz[j] - s.z) + (T)(lz[j] - l.z), nx[j], ny[j], nz[j], mx,
-                                                    my, mz, wv, s_exp, l_exp, pt[j]);
+                                                    my, mz, wv, s_exp, l_exp, pt[j], rp);
                 }
             } else {
 #pragma unroll 2
@@ -1044,7 +1162,7 @@ k_apply(const typename V4T<T>::type* __restrict__ fa, const typename V4T<T>::typ
 #pragma unroll
                     for (int j = 0; j < TT; ++j)
                         apply_term<T, OP, false, KC>(tx[j] - s.x, ty[j] - s.y, tz[j] - s.z, nx[j], ny[j], nz[j],
-                                                     mx, my, mz, wv, s_exp, l_exp, pt[j]);
+                                                     mx, my, mz, wv, s_exp, l_exp, pt[j], rp);
                 }
             }
 #pragma unroll
@@ -1510,6 +1628,28 @@ k_apply_combine(const double* __restrict__ part, int nsplit, int nf, const d4* _
     }
 }
 
+// the FP64 power plan of |d|^{-2s}, s = 2 - 2/p (or, for L, of |d|^{-2(1 + 2/p)}):
+// rational when 2 n / p is a whole number for some n <= 16 (p = 6: n = 3; 4.5: n = 9)
+static RootPow root_plan(double p, bool op_l) {
+    RootPow r;
+    const double q = 2.0 / p;
+    r.a = op_l ? 3.0 - (2.0 - q) : 2.0 - q;
+    for (int n = 1; n <= 16; ++n) {
+        const double m = std::round(q * n);
+        if (std::fabs(q * n - m) > 4e-16 * n) continue;
+        const int k = op_l ? n + (int)m : 2 * n - (int)m;
+        r.n = n;
+        r.k = k;
+        r.a = (double)k / n;
+        r.inv = -1.f / (float)n;
+        break;
+    }
+    r.c1 = r.a;
+    r.c2 = 0.5 * r.a * (r.a + 1.0);
+    r.c3 = r.a * (r.a + 1.0) * (r.a + 2.0) / 6.0;
+    return r;
+}
+
 template <typename T, int OP, int KC>
 static int launch_apply_op(tp_mesh* m, const tp_params* p, const double* v, int k, double* y,
                            cudaStream_t st) {
@@ -1520,6 +1660,7 @@ static int launch_apply_op(tp_mesh* m, const tp_params* p, const double* v, int 
     const double l_exp = 3.0 - s;            // |d|^{-(2 sigma + 2)} = r2^{-(sigma+1)}, sigma = 2 - s
     constexpr int TT = (sizeof(T) == 4 && KC == 3) ? 2 : 1;
     Grid g = make_grid(nf, nf, TT, resident_per_sm((const void*)k_apply<T, OP, TT, KC>, NT));
+    if (sizeof(T) == 8) g = fp64_grid(g, nf);
     TP_TRY(ensure(m->part, sizeof(double) * (size_t)g.nsplit * L::NA * nf));
     TP_TRY(ensure(m->wv64, sizeof(double) * 4 * KC * (size_t)nf));
     TP_TRY(ensure(m->wv32, sizeof(V4) * L::NW4 * (size_t)nf));
@@ -1539,9 +1680,10 @@ static int launch_apply_op(tp_mesh* m, const tp_params* p, const double* v, int 
                               : OP == TP_OP_B0 ? PK_APPLY_B0 : PK_APPLY_L;
             ProfScope ps(m, key, units, st);
             m->prof.cols[key] += KC;
-            k_apply<T, OP, TT, KC><<<grid, NT, 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
+            k_apply<T, OP, TT, KC><<<grid, NT, sizeof(T) == 8 ? two_resident(k_apply<T, OP, TT, KC>) : 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
                                                         m->center.as<double>(), m->wv32.as<V4>(), nf,
-                                                        g.tiles_per_split, T(s), T(l_exp), m->part.as<double>());
+                                                        g.tiles_per_split, T(s), T(l_exp), m->part.as<double>(),
+                                                        root_plan(p->p, OP == TP_OP_L));
         }
         TP_LAUNCH_CHECK();
         k_apply_combine<OP, KC><<<(nf + 31) / 32, dim3(32, KC + 1), 0, st>>>(m->part.as<double>(), g.nsplit, nf,
