@@ -5,12 +5,12 @@
 // (host, once per topology). Per set of positions the values of C change and
 // the factor is recomputed:
 //
-//   factor (one launch per tree level, one block per supernode J): assemble
-//   the panel (t x nJ, shared memory) from the entries of C in J's columns and
-//   the children's update matrices, factor its diagonal block (right-looking,
-//   column by column), form U_J = (children's share of struct x struct) -
-//   L21 L21^T (global memory), and store L11^-1 (explicit inverse of the
-//   diagonal block) and L21.
+//   factor (two launches per tree level): k_chol_panel, one block per supernode
+//   J, assembles the panel (t x nJ, shared memory) from the entries of C in J's
+//   columns and the children's update matrices, factors its diagonal block
+//   (right-looking, column by column) with L11^-1 formed along the way, and
+//   stores L11^-1 and L21; k_chol_update, one block per 64 x 64 tile, forms
+//   U_J = (children's share of struct x struct) - L21 L21^T (global memory).
 //
 //   solve (forward levels leaves -> root, backward levels root -> leaves):
 //   with L11^-1 stored, each supernode's step is two small dense mat-vecs on
@@ -34,25 +34,32 @@ namespace tp {
 
 constexpr int CH_KMAX = 9;
 constexpr int CH_LEAF = 64;                    // vertices per leaf supernode
-constexpr int CHF_T = 256;                     // factor block
+constexpr int CHF_TILE = 64;                   // tile of an update matrix (k_chol_update)
+constexpr int CHF_KC = 32;                     // columns of L21 staged at a time
 constexpr int CHS_T = 256;                     // solve block
 constexpr int CHR_T = 256;                     // residual block
-constexpr size_t CH_SMEM_MAX = 200 * 1024;     // largest factor panel kept in shared memory
+constexpr size_t CHS_SMALL = 70 * 1024;        // solve step of which an SM holds three blocks
+constexpr size_t CH_SMEM_MAX = 220 * 1024;     // dynamic shared memory of a factor panel or a solve step
 
 struct CholNode {   // 64 bytes
     int p0, nJ, mJ, t;
     long long loff, uoff;
     int voff, child0, child1, s0;
-    int asm0, asm1, pad0, pad1;
+    int asm0, asm1, ldu, flags;   // leading dimension of U
 };
 static_assert(sizeof(CholNode) == 64, "CholNode layout");
+// the node's one child has exactly the rows of its front: its U is the trailing
+// part of the child's U, updated in place (the links of a separator's chain)
+constexpr int CHN_INPLACE = 1;
+// the children's update vectors are read from global memory in the solve
+constexpr int CHN_DIRECT = 2;
 
 struct CholCtl {
     int done;       // 1: every column converged (or the refinement gave up)
     int stalled;    // 1: the residual stopped decreasing
     int iters;      // refinement sweeps done
     int err;        // 1: a cross-block wait of a sweep gave up
-    unsigned ticket, bcount, arrive;   // sweep scheduling (zero between sweeps)
+    unsigned ticket[3], bcount, arrive;   // sweep scheduling (zero between sweeps)
     int bad_pivot;  // 1: a non-positive pivot appeared in the factorisation
     double bb[CH_KMAX], rr[CH_KMAX];
     unsigned epoch;  // sweeps finished; never cleared (the node flags compare against it)
@@ -64,12 +71,17 @@ struct CholState {
     std::string why;
     int H = 0;                            // number of levels
     std::vector<int> lvl_max_t, lvl_max_n, lvl_max_m;
-    std::vector<size_t> lvl_factor_smem, lvl_solve_smem;   // bytes; solve: factor block + 9-column vectors
+    std::vector<size_t> lvl_factor_smem;  // bytes
+    std::vector<int> lvl_tile;            // first entry of each level in `tiles`
     std::vector<double> lvl_factor_flops;
     double solve_bytes = 0.0;             // factor bytes read by one forward + backward sweep
     Buf nodes, level_nodes, child_idx, rel, struct_pos, asm_dst, asm_src, perm, comp_ptr, comp_verts, comp_of;
-    Buf parent, fdone, bdone, trace;
-    size_t solve_smem = 0;     // dynamic shared memory of the sweep kernel
+    Buf parent, fdone, bdone, trace, tiles;
+    // dynamic shared memory of the sweep kernel by column count: the largest of all
+    // nodes, and of the leading tree levels that leave room for three blocks per SM
+    // (small_n nodes, small_lvls levels)
+    size_t solve_smem[CH_KMAX + 1] = {}, small_smem[CH_KMAX + 1] = {};
+    int small_n[CH_KMAX + 1] = {};
     Buf L, U, uvec, ybuf, xbuf, ctl, part, x, r, bp;
     bool factored = false;
     int ncomp = 1;
@@ -93,97 +105,286 @@ struct CholState {
 // factorisation
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(CHF_T)
-k_chol_factor(const CholNode* __restrict__ nodes, const int* __restrict__ lvl, const int* __restrict__ child_idx,
-              const int* __restrict__ rel, const int* __restrict__ asm_dst, const int* __restrict__ asm_src,
-              const double* __restrict__ val, float* __restrict__ L, float* __restrict__ U,
-              CholCtl* __restrict__ ctl) {
-    extern __shared__ float smem[];
-    __shared__ float s_rd;
+// Panel of one supernode per block: assembly, Cholesky of the diagonal block
+// and its inverse, in blocks of CHF_NB columns. Latency-bound: the blocks of
+// columns come one after the other, and the levels above the leaves hold fewer
+// supernodes than the GPU has SMs. Hence few barriers (three per block of
+// columns: every thread factors the CHF_NB x CHF_NB diagonal block for itself
+// and substitutes into its own rows), and a trailing update of rank CHF_NB with
+// the row factors in registers, which takes the remaining panel columns and the
+// columns of L11^-1 alike (the same row operations on the identity). 25,000
+// vertices, 9 levels: 31 us a level on average, 84 us one column at a time.
+constexpr int CHF_NB = 8;
+
+// shared floats of a panel of t rows and n columns: P (t x n), X (n x n, leading
+// dimension a multiple of 8), the block's rows below it (n x NB), the rows of the
+// largest child
+__host__ __device__ inline int chf_ldx(int n) { return (n + CHF_NB - 1) / CHF_NB * CHF_NB; }
+inline size_t chf_smem(size_t t, size_t n, size_t child) {
+    return sizeof(float) * (((t * n + 3) & ~size_t(3)) + (size_t)chf_ldx((int)n) * n + chf_ldx((int)n) * CHF_NB + child);
+}
+
+__global__ void __launch_bounds__(512)
+k_chol_panel(const CholNode* __restrict__ nodes, const int* __restrict__ lvl, const int* __restrict__ child_idx,
+             const int* __restrict__ rel, const int* __restrict__ asm_dst, const int* __restrict__ asm_src,
+             const double* __restrict__ val, float* __restrict__ L, const float* __restrict__ U,
+             CholCtl* __restrict__ ctl) {
+    constexpr int NB = CHF_NB;
+    extern __shared__ float4 smem4_f[];
+    float* smem = reinterpret_cast<float*>(smem4_f);
     const CholNode nd = nodes[lvl[blockIdx.x]];
     const int n = nd.nJ, m = nd.mJ, t = nd.t;
-    float* P = smem;                 // panel t x n, column-major
-    float* X = smem + (size_t)t * n; // L11^-1, n x n column-major
-    float* UJ = U + nd.uoff;         // m x m, column-major (lower part used)
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = CHF_T / 32;
+    const int ldx = chf_ldx(n);
+    float* P = smem;                                   // panel t x n, column-major
+    float* X = smem + ((t * n + 3) & ~3);              // L11^-1, n columns, leading dimension ldx
+    float* B = X + (size_t)ldx * n;                    // rows of the block's L: B[row][NB]
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = tid >> 5, NW = T >> 5;
 
-    for (int i = tid; i < t * n; i += CHF_T) P[i] = 0.f;
-    for (int i = tid; i < m * m; i += CHF_T) UJ[i] = 0.f;
+    if (nd.flags & CHN_INPLACE) {
+        // the panel is the first n columns of the child's update matrix
+        const float* Uc = U + nodes[child_idx[nd.child0]].uoff;
+        for (int y = warp; y < n; y += NW)
+#pragma unroll 8
+            for (int x = lane; x < t; x += 32) P[x + y * t] = x >= y ? Uc[x + (size_t)y * nd.ldu] : 0.f;
+    } else {
+        for (int i = tid; i < t * n; i += T) P[i] = 0.f;
+    }
+    for (int i = tid; i < ldx * n; i += T) X[i] = i % ldx == i / ldx ? 1.f : 0.f;
+    for (int i = tid; i < ldx * NB; i += T) B[i] = 0.f;
     __syncthreads();
     // entries of C in J's columns (each panel position at most once)
-    for (int e = nd.asm0 + tid; e < nd.asm1; e += CHF_T) P[asm_dst[e]] = (float)val[asm_src[e]];
+    for (int e = nd.asm0 + tid; e < nd.asm1; e += T) P[asm_dst[e]] += (float)val[asm_src[e]];
     __syncthreads();
-    // extend-add of the children's update matrices, one child at a time
-    for (int ci = nd.child0; ci < nd.child1; ++ci) {
-        const CholNode cn = nodes[child_idx[ci]];
-        const int mc = cn.mJ;
-        const int* rl = rel + cn.s0;
-        const float* Uc = U + cn.uoff;
-        for (int idx = tid; idx < mc * mc; idx += CHF_T) {
-            const int y = idx / mc, x = idx - y * mc;
-            if (x < y) continue;
-            const int R = rl[x], Cc = rl[y];
-            const float v = Uc[idx];
-            if (Cc < n)
-                P[R + Cc * t] += v;
-            else
-                UJ[(R - n) + (Cc - n) * m] += v;
+    if (!(nd.flags & CHN_INPLACE)) {
+        // extend-add of the children's columns that fall into the panel (the
+        // first ones: a child's rows are sorted), one child at a time, its rows'
+        // places in the front staged first
+        int* rl = reinterpret_cast<int*>(B + ldx * NB);
+        for (int ci = nd.child0; ci < nd.child1; ++ci) {
+            const CholNode cn = nodes[child_idx[ci]];
+            const int mc = cn.mJ;
+            const float* Uc = U + cn.uoff;
+            for (int x = tid; x < mc; x += T) rl[x] = rel[cn.s0 + x];
+            __syncthreads();
+            int lo = 0, hi = mc;     // columns with a place before n
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (rl[mid] < n) lo = mid + 1;
+                else hi = mid;
+            }
+            const int cnt = lo * mc;
+            for (int e0 = tid; e0 < cnt; e0 += 4 * T) {
+                float v[4];
+                int at[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int e = e0 + q * T, y = e / mc, x = e - y * mc;
+                    at[q] = -1;
+                    if (e < cnt && x >= y) {
+                        v[q] = Uc[x + (size_t)y * cn.ldu];
+                        at[q] = rl[x] + rl[y] * t;
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (at[q] >= 0) P[at[q]] += v[q];
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
-    // right-looking Cholesky of the diagonal block; the rows below it become L21
-    for (int k = 0; k < n; ++k) {
-        if (tid == 0) {
-            float d = P[k + k * t];
+    for (int kb = 0; kb < n; kb += NB) {
+        const int nb = min(NB, n - kb);
+        // the diagonal block (columns past n: identity), factored by every thread;
+        // D[k][l] = L entries below the diagonal, rd = reciprocal diagonal
+        float D[NB][NB], rd[NB];
+#pragma unroll
+        for (int l = 0; l < NB; ++l)
+#pragma unroll
+            for (int k = l; k < NB; ++k) D[k][l] = k < nb ? P[kb + k + (kb + l) * t] : (k == l ? 1.f : 0.f);
+        bool bad = false;
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+            float d = D[k][k];
             if (!(d > 0.f)) {
-                ctl->bad_pivot = 1;
+                bad = true;
                 d = 1.f;
             }
-            d = sqrtf(d);
-            P[k + k * t] = d;
-            s_rd = 1.f / d;
+            // correctly rounded steps: rsqrtf with a Newton step made the refinement
+            // take a sweep more (163,842 vertices)
+            rd[k] = 1.f / sqrtf(d);
+#pragma unroll
+            for (int i = k + 1; i < NB; ++i) D[i][k] *= rd[k];
+#pragma unroll
+            for (int j = k + 1; j < NB; ++j)
+#pragma unroll
+                for (int i = j; i < NB; ++i) D[i][j] = fmaf(-D[i][k], D[j][k], D[i][j]);
+        }
+        if (bad && tid == 0) ctl->bad_pivot = 1;
+        // rows below the block: substitution, row by row; rows of the diagonal
+        // block's own columns go to B too
+        for (int i = kb + nb + tid; i < t; i += T) {
+            float r[NB];
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
+                float x = k < nb ? P[i + (kb + k) * t] : 0.f;
+#pragma unroll
+                for (int l = 0; l < k; ++l) x = fmaf(-r[l], D[k][l], x);
+                r[k] = x * rd[k];
+            }
+#pragma unroll
+            for (int k = 0; k < NB; ++k)
+                if (k < nb) P[i + (kb + k) * t] = r[k];
+            if (i < n) {
+                float4* br = reinterpret_cast<float4*>(B + i * NB);
+                br[0] = make_float4(r[0], r[1], r[2], r[3]);
+                br[1] = make_float4(r[4], r[5], r[6], r[7]);
+            }
+        }
+        // the block's rows of the inverse: X_b <- L_bb^-1 X_b, a thread per column
+        for (int c = T - 1 - tid; c < kb + nb; c += T) {
+            float4* xc = reinterpret_cast<float4*>(X + kb + (size_t)c * ldx);
+            const float4 x0 = xc[0], x1 = xc[1];
+            float r[NB] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
+                float x = r[k];
+#pragma unroll
+                for (int l = 0; l < k; ++l) x = fmaf(-r[l], D[k][l], x);
+                r[k] = x * rd[k];
+            }
+            xc[0] = make_float4(r[0], r[1], r[2], r[3]);
+            xc[1] = make_float4(r[4], r[5], r[6], r[7]);
         }
         __syncthreads();
-        const float rd = s_rd;
-        for (int i = k + 1 + tid; i < t; i += CHF_T) P[i + k * t] *= rd;
-        __syncthreads();
-        for (int j = k + 1 + warp; j < n; j += NW) {
-            const float ljk = P[j + k * t];
-            for (int i = j + lane; i < t; i += 32) P[i + j * t] -= P[i + k * t] * ljk;
+        const int k1 = kb + nb;
+        if (k1 >= n) break;
+        // trailing update: work items are (32 rows, eight columns); panel columns
+        // k1 .. n with all rows from k1, inverse columns 0 .. k1 with rows k1 .. n
+        const int pch = (t - k1 + 31) / 32, pgr = (n - k1 + 7) / 8;
+        const int xch = (n - k1 + 31) / 32, xgr = (k1 + 7) / 8;
+        const int items = pch * pgr + xch * xgr;
+        for (int w = warp; w < items; w += NW) {
+            const bool inv = w >= pch * pgr;
+            const int q = inv ? w - pch * pgr : w, ch = inv ? xch : pch;
+            const int i = k1 + (q % ch) * 32 + lane, j0 = (inv ? 0 : k1) + (q / ch) * 8;
+            const int iend = inv ? n : t, jend = inv ? k1 : n;
+            if (i >= iend) continue;
+            float r[NB];
+#pragma unroll
+            for (int k = 0; k < NB; ++k) r[k] = k < nb ? P[i + (kb + k) * t] : 0.f;
+            float* out = inv ? X + i : P + i;
+            const int ldo = inv ? ldx : t;
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) {
+                const int j = j0 + jj;
+                if (j < jend) {
+                    const float4* bj = reinterpret_cast<const float4*>(inv ? X + kb + (size_t)j * ldx : B + j * NB);
+                    const float4 b0 = bj[0], b1 = bj[1];
+                    float x = out[(size_t)j * ldo];
+                    x = fmaf(-r[0], b0.x, x);
+                    x = fmaf(-r[1], b0.y, x);
+                    x = fmaf(-r[2], b0.z, x);
+                    x = fmaf(-r[3], b0.w, x);
+                    x = fmaf(-r[4], b1.x, x);
+                    x = fmaf(-r[5], b1.y, x);
+                    x = fmaf(-r[6], b1.z, x);
+                    x = fmaf(-r[7], b1.w, x);
+                    out[(size_t)j * ldo] = x;
+                }
+            }
         }
         __syncthreads();
     }
-    // U_J -= L21 L21^T (lower part)
-    for (int idx = tid; idx < m * m; idx += CHF_T) {
-        const int y = idx / m, x = idx - y * m;
-        if (x < y) continue;
-        float s = 0.f;
-        for (int k = 0; k < n; ++k) s += P[n + x + k * t] * P[n + y + k * t];
-        UJ[idx] -= s;
-    }
-    // X = L11^-1 by forward substitution, one column per thread
-    for (int c = tid; c < n; c += CHF_T) {
-        for (int i = 0; i < c; ++i) X[i + c * n] = 0.f;
-        X[c + c * n] = 1.f / P[c + c * t];
-        for (int i = c + 1; i < n; ++i) {
-            float s = 0.f;
-            for (int k = c; k < i; ++k) s += P[i + k * t] * X[k + c * n];
-            X[i + c * n] = -s / P[i + i * t];
-        }
-    }
-    __syncthreads();
     const int ldn = n | 1, ldm = m == 0 ? 0 : (m | 1);
     float* Lj = L + nd.loff;   // n x n, leading dimension ldn
-    for (int i = tid; i < n * n; i += CHF_T) {
-        const int c = i / n, r = i - c * n;
-        Lj[r + c * ldn] = X[i];
-    }
     float* L21 = Lj + (size_t)n * ldn;   // m x n, leading dimension ldm
-    for (int idx = tid; idx < m * n; idx += CHF_T) {
-        const int k = idx / m, x = idx - k * m;
-        L21[x + k * ldm] = P[n + x + k * t];
+    for (int c = warp; c < n; c += NW) {
+        for (int r = lane; r < n; r += 32) Lj[r + c * ldn] = r >= c ? X[r + c * ldx] : 0.f;
+        for (int x = lane; x < m; x += 32) L21[x + c * ldm] = P[n + x + c * t];
     }
+}
+
+// A 64 x 64 tile (lower part) of one supernode's update matrix: the children's
+// entries that fall into it (contiguous row and column ranges of each child,
+// whose rows are sorted; in place: the tile itself), minus L21 L21^T. tiles:
+// (node, first row, first column). A level's tiles run side by side (12 us a level
+// on 25,000 vertices, mostly its chain of dependent loads); one block per supernode
+// did this work and the panel in 127 us.
+__global__ void __launch_bounds__(256)
+k_chol_update(const CholNode* __restrict__ nodes, const int4* __restrict__ tiles, const int* __restrict__ child_idx,
+              const int* __restrict__ rel, const float* __restrict__ L, float* __restrict__ U) {
+    constexpr int TB = CHF_TILE, KC = CHF_KC;
+    __shared__ float S[TB][TB + 1];          // [column][row]
+    __shared__ __align__(16) float As[KC][TB], Bs[KC][TB];
+    __shared__ int s_rng[4];
+    const int4 tl = tiles[blockIdx.x];
+    const CholNode nd = nodes[tl.x];
+    const int n = nd.nJ, m = nd.mJ, r0 = tl.y, c0 = tl.z, tid = threadIdx.x;
+    const int rn = min(TB, m - r0), cn = min(TB, m - c0);
+    const int ldm = m | 1;
+    const float* L21 = L + nd.loff + (size_t)n * (n | 1);
+    float* UJ = U + nd.uoff;
+    const bool inplace = nd.flags & CHN_INPLACE;
+    if (!inplace) {
+        for (int i = tid; i < TB * (TB + 1); i += 256) (&S[0][0])[i] = 0.f;
+        __syncthreads();
+        for (int ci = nd.child0; ci < nd.child1; ++ci) {
+            const CholNode ch = nodes[child_idx[ci]];
+            const int* rl = rel + ch.s0;
+            if (tid < 4) {   // first child row at or after front rows n + r0, n + r0 + rn, n + c0, n + c0 + cn
+                const int want = n + (tid == 0 ? r0 : tid == 1 ? r0 + rn : tid == 2 ? c0 : c0 + cn);
+                int lo = 0, hi = ch.mJ;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (rl[mid] < want) lo = mid + 1;
+                    else hi = mid;
+                }
+                s_rng[tid] = lo;
+            }
+            __syncthreads();
+            const int x0 = s_rng[0], x1 = s_rng[1], y0 = s_rng[2], y1 = s_rng[3];
+            const float* Uc = U + ch.uoff;
+            for (int y = y0 + (tid >> 5); y < y1; y += 8) {
+                const int c = rl[y] - n - c0;
+                for (int x = max(x0, y) + (tid & 31); x < x1; x += 32) S[c][rl[x] - n - r0] += Uc[x + (size_t)y * ch.ldu];
+            }
+            __syncthreads();
+        }
+    }
+    const int tx = tid & 15, ty = tid >> 4;   // rows tx + 16 i, columns 4 ty + j
+    float acc[4][4] = {};
+    for (int k0 = 0; k0 < n; k0 += KC) {
+        const int kn = min(KC, n - k0);
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < KC * TB / 256; ++u) {
+            const int i = tid + u * 256, k = i / TB, r = i % TB;
+            As[k][r] = k < kn && r < rn ? L21[r0 + r + (size_t)(k0 + k) * ldm] : 0.f;
+            Bs[k][r] = k < kn && r < cn ? L21[c0 + r + (size_t)(k0 + k) * ldm] : 0.f;
+        }
+        __syncthreads();
+        const int ke = (kn + 7) & ~7;
+#pragma unroll 8
+        for (int k = 0; k < ke; ++k) {
+            const float4 b = *reinterpret_cast<const float4*>(&Bs[k][4 * ty]);
+            const float bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float av = As[k][tx + 16 * i];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av, bv[j], acc[i][j]);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = tx + 16 * i, c = 4 * ty + j;
+            if (r >= rn || c >= cn || r0 + r < c0 + c) continue;
+            float* u = UJ + (r0 + r) + (size_t)(c0 + c) * nd.ldu;
+            *u = (inplace ? *u : S[c][r]) - acc[i][j];
+        }
 }
 
 // ---------------------------------------------------------------------------
@@ -228,6 +429,7 @@ struct SweepArgs {
     unsigned long long* trace;   // per ticket timestamps (builds with TP_CHOL_TRACE only)
     double tol2;
     int nv, nn, cap;
+    int phase, t0, t1, last;  // this launch's part of the sweep: tickets t0 .. t1, and whether the residual follows
 };
 
 #ifdef TP_CHOL_TRACE
@@ -333,6 +535,80 @@ __device__ __forceinline__ void rows_matvec(const float* M, int sr, int sk, int 
     }
 }
 
+// rows_matvec of mode 2 for many rows and few terms (a wide front's L21 y): every
+// thread takes four rows at a time, which share the broadcast reads of v
+template <int K, class Out>
+__device__ __forceinline__ void tall_matvec(const float* M, int ld, int R, int n, const float* v, Out out) {
+    constexpr int KP = Kp<K>::P, RT = 4;
+    for (int r0 = threadIdx.x; r0 < R; r0 += CHS_T * RT) {
+        float acc[RT][K];
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+#pragma unroll
+            for (int c = 0; c < K; ++c) acc[i][c] = 0.f;
+#pragma unroll 2
+        for (int k = 0; k < n; ++k) {
+            float vk[KP];
+#pragma unroll
+            for (int q = 0; q < KP / 4; ++q) {
+                const float4 t = reinterpret_cast<const float4*>(v + k * KP)[q];
+                vk[4 * q] = t.x; vk[4 * q + 1] = t.y; vk[4 * q + 2] = t.z; vk[4 * q + 3] = t.w;
+            }
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                const int r = r0 + i * CHS_T;
+                const float mr = r < R ? M[r + k * ld] : 0.f;
+#pragma unroll
+                for (int c = 0; c < K; ++c) acc[i][c] = fmaf(mr, vk[c], acc[i][c]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+            if (r0 + i * CHS_T < R) out(r0 + i * CHS_T, acc[i]);
+    }
+    __syncthreads();
+}
+
+// out(r, acc) with acc[c] = sum_{k < n} M[r * ld + k] v[k][c] for few rows of many
+// terms (a wide front's L21^T x): the lanes of a warp share a row's terms, in two
+// rows at a time, and add up by a fixed butterfly. rows_matvec kept two threads a
+// row busy here: 8 us a step for 24 rows of 1,000 terms.
+template <int K, class Out>
+__device__ __forceinline__ void wide_matvec(const float* M, int ld, int R, int n, const float* v, Out out) {
+    constexpr int KP = Kp<K>::P, RT = 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int r0 = warp * RT; r0 < R; r0 += (CHS_T / 32) * RT) {
+        float acc[RT][K];
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+#pragma unroll
+            for (int c = 0; c < K; ++c) acc[i][c] = 0.f;
+#pragma unroll 2
+        for (int k = lane; k < n; k += 32) {
+            float vk[KP];
+#pragma unroll
+            for (int q = 0; q < KP / 4; ++q) {
+                const float4 t = reinterpret_cast<const float4*>(v + k * KP)[q];
+                vk[4 * q] = t.x; vk[4 * q + 1] = t.y; vk[4 * q + 2] = t.z; vk[4 * q + 3] = t.w;
+            }
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                const float mr = r0 + i < R ? M[(r0 + i) * ld + k] : 0.f;
+#pragma unroll
+                for (int c = 0; c < K; ++c) acc[i][c] = fmaf(mr, vk[c], acc[i][c]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+#pragma unroll
+            for (int c = 0; c < K; ++c)
+                for (int o = 16; o > 0; o >>= 1) acc[i][c] += __shfl_xor_sync(0xffffffffu, acc[i][c], o);
+            if (lane == 0 && r0 + i < R) out(r0 + i, acc[i]);
+        }
+    }
+    __syncthreads();
+}
+
 // shared-memory layout of a solve step (floats): factor block, then the
 // K-column vectors (rows of KP floats): forward w (t), y (n); backward x_S
 // (m), y_J (n), z (n); then the two-half scratch (128 rows); then (backward)
@@ -370,7 +646,7 @@ __device__ __forceinline__ void fwd_prepare(const SweepArgs& A, const CholNode& 
                       [&](int e) { const int a = e / K; return a < n ? (float)__ldcg(A.r + (size_t)perm[a] * K + (e - a * K)) : 0.f; },
                       [&](int e, float v) { const int a = e / K; w[a * KP + (e - a * K)] = v; });
     const int nc = nd.child1 - nd.child0;
-    if (nc <= CH_MAXCH) {
+    if (nc <= CH_MAXCH && !(nd.flags & CHN_DIRECT)) {
         // the children's records, then their target rows in this front
         if (tid == 0) {
             int row0 = 0;
@@ -399,7 +675,7 @@ __device__ void fwd_finish(const SweepArgs& A, const CholNode& nd, float* smem, 
     const float* Li = smem;       // n x n, leading dimension ldn
     const float* L21 = smem + n * ldn;   // m x n, leading dimension ldm
     const int nc = nd.child1 - nd.child0;
-    if (nc <= CH_MAXCH) {
+    if (nc <= CH_MAXCH && !(nd.flags & CHN_DIRECT)) {
         // every child's update vector in one batched pass, then the
         // extend-add from shared memory, one child at a time
         const int rows = nc ? kids[nc - 1].row0 + kids[nc - 1].mJ : 0;
@@ -427,10 +703,12 @@ __device__ void fwd_finish(const SweepArgs& A, const CholNode& nd, float* smem, 
             const CholNode cn = A.nodes[A.child_idx[nd.child0 + ci]];
             const int* rl = A.rel + cn.s0;
             const float* uc = A.uvec + (size_t)cn.voff * K;
-            for (int idx = tid; idx < cn.mJ * K; idx += CHS_T) {
-                const int x = idx / K, c = idx - x * K;
-                w[rl[x] * KP + c] += __ldcg(uc + idx);
-            }
+            const bool same = nd.flags & CHN_INPLACE;   // the child's rows are this front's
+            gather_batched<12>(cn.mJ * K, [&](int e) { return __ldcg(uc + e); },
+                               [&](int e, float v) {
+                                   const int x = e / K;
+                                   w[(same ? x : __ldg(rl + x)) * KP + (e - x * K)] += v;
+                               });
             __syncthreads();
         }
     }
@@ -443,10 +721,15 @@ __device__ void fwd_finish(const SweepArgs& A, const CholNode& nd, float* smem, 
         }
     });
     float* uj = A.uvec + (size_t)nd.voff * K;
-    rows_matvec<K>(L21, 1, ldm, m, n, 2, y, sm.scratch, [&](int r, const float (&acc)[K]) {
+    auto put_u = [&](int r, const float (&acc)[K]) {
 #pragma unroll
         for (int c = 0; c < K; ++c) uj[r * K + c] = w[(n + r) * KP + c] - acc[c];
-    });
+    };
+    // (two passes of 128 rows or fewer keep both halves of the block on a row)
+    if (m > 256)
+        tall_matvec<K>(L21, ldm, m, n, y, put_u);
+    else
+        rows_matvec<K>(L21, 1, ldm, m, n, 2, y, sm.scratch, put_u);
 }
 
 // backward step of node J. bwd_prepare stages the factor block and the
@@ -494,10 +777,16 @@ __device__ void bwd_finish(const SweepArgs& A, const CholNode& nd, float* smem) 
                           }
                       });
     __syncthreads();
-    rows_matvec<K>(L21, ldm, 1, n, m, 2, xs, sm.scratch, [&](int r, const float (&acc)[K]) {
+    auto put_z = [&](int r, const float (&acc)[K]) {
 #pragma unroll
         for (int c = 0; c < K; ++c) z[r * KP + c] = yj[r * KP + c] - acc[c];
-    });
+    };
+    // rows_matvec takes about 15 cycles per term of its longest thread, m / 2 terms;
+    // the lanes' sums about 30 per column and row, n / 8 rows a warp
+    if (m > 4 * n && m > 128)
+        wide_matvec<K>(L21, ldm, n, m, xs, put_z);
+    else
+        rows_matvec<K>(L21, ldm, 1, n, m, 2, xs, sm.scratch, put_z);
     float* xb = A.xbuf + (size_t)nd.p0 * K;
     const double* xo = sm.xo;
     rows_matvec<K>(Li, ldn, 1, n, n, 1, z, sm.scratch, [&](int r, const float (&acc)[K]) {
@@ -564,15 +853,16 @@ k_chol_sweep(SweepArgs A) {
     __shared__ double s_red[CHS_T];
     const unsigned ep = *(volatile unsigned*)&ctl->epoch + 1;
     const int nn = A.nn, tid = threadIdx.x;
-    if (tid == 0) s_tk = (int)atomicAdd(&ctl->ticket, 1u);
+    unsigned* ticket = &ctl->ticket[A.phase];
+    if (tid == 0) s_tk = A.t0 + (int)atomicAdd(ticket, 1u);
     __syncthreads();
     for (;;) {
         const int tk = s_tk;
-        if (tk >= 2 * nn) break;
+        if (tk >= A.t1) break;
         // the next ticket is taken now and used after this step: the atomic's
         // latency overlaps the step (the block runs both steps in order)
         unsigned next = 0;
-        if (tid == 0) next = atomicAdd(&ctl->ticket, 1u);
+        if (tid == 0) next = A.t0 + atomicAdd(ticket, 1u);
         const bool fwd = tk < nn;
         CH_TRACE(tk, 0);
         const int J = fwd ? A.order[tk] : A.order[2 * nn - 1 - tk];
@@ -618,6 +908,7 @@ k_chol_sweep(SweepArgs A) {
         }
         __syncthreads();
     }
+    if (!A.last) return;
     // r = bp - C x once every backward step is done; per-block sums of r.r
     CH_TRACE(2 * nn + blockIdx.x, 0);
     if (tid == 0) s_ok = wait_until(&ctl->bcount, (unsigned)nn, true, ctl);
@@ -689,7 +980,7 @@ k_chol_sweep(SweepArgs A) {
             ctl->stalled = 1;
         }
         CH_TRACE(2 * nn + gridDim.x, 0);
-        ctl->ticket = 0;
+        ctl->ticket[0] = ctl->ticket[1] = ctl->ticket[2] = 0;
         ctl->arrive = 0;
         ctl->bcount = 0;
         __threadfence();
@@ -860,7 +1151,7 @@ void chol_release(tp_mesh* m) {
     CholState* c = m->chol;
     Buf* all[] = {&c->nodes, &c->level_nodes, &c->child_idx, &c->rel, &c->struct_pos, &c->asm_dst,
                   &c->asm_src, &c->perm, &c->comp_ptr, &c->comp_verts, &c->comp_of, &c->parent, &c->fdone,
-                  &c->bdone, &c->L, &c->U,
+                  &c->bdone, &c->tiles, &c->L, &c->U,
                   &c->uvec, &c->ybuf, &c->xbuf, &c->ctl, &c->part, &c->x, &c->r, &c->bp, &c->dflags};
     for (Buf* b : all) release(*b);
     for (auto& g : c->graph)
@@ -926,42 +1217,86 @@ static int chol_setup(tp_mesh* m) {
     c->lvl_max_n.assign(c->H, 0);
     c->lvl_max_m.assign(c->H, 0);
     c->lvl_factor_smem.assign(c->H, 0);
-    c->lvl_solve_smem.assign(c->H, 0);
     c->lvl_factor_flops.assign(c->H, 0.0);
+    // bytes of a solve step on K columns: the factor block (rounded to 16 bytes),
+    // the vectors (rows of K rounded to whole float4s), the 128-row scratch, the
+    // node's FP64 solution entries, then struct(J) or the staged rows and update
+    // vectors of the children (see StepSmem)
+    auto step_smem = [&](int J, int K, bool direct) {
+        const size_t n = S.nJ[J], mm = S.mJ[J], KP = (K + 3) & ~3;
+        size_t csum = 0;   // rows of the children's update vectors
+        if (!direct)
+            for (int ci = S.child_ptr[J]; ci < S.child_ptr[J + 1]; ++ci) csum += S.mJ[S.child_idx[ci]];
+        return sizeof(float) * (((n * chol_ld(n) + n * chol_ld(mm) + 3) & ~size_t(3)) + (mm + 2 * n) * KP + 128 * KP +
+                                2 * n * K + std::max(csum * (K + 1), mm) + 4);
+    };
     size_t worst = 0;
-    for (int h = 0; h < c->H; ++h)
+    bool small_open[CH_KMAX + 1];
+    std::fill(small_open, small_open + CH_KMAX + 1, true);
+    std::vector<int> flags(S.nnode, 0);
+    for (int h = 0; h < c->H; ++h) {
+        size_t lvl_smem[CH_KMAX + 1] = {};
         for (int i = S.level_ptr[h]; i < S.level_ptr[h + 1]; ++i) {
             const int J = S.level_nodes[i];
             const double n = S.nJ[J], mm = S.mJ[J];
             c->lvl_max_t[h] = std::max(c->lvl_max_t[h], S.nJ[J] + S.mJ[J]);
             c->lvl_max_n[h] = std::max(c->lvl_max_n[h], S.nJ[J]);
             c->lvl_max_m[h] = std::max(c->lvl_max_m[h], S.mJ[J]);
-            const size_t sm = sizeof(float) * ((size_t)(S.nJ[J] + S.mJ[J]) * S.nJ[J] + (size_t)S.nJ[J] * S.nJ[J]);
+            int child = 0;   // rows of the largest child
+            for (int ci = S.child_ptr[J]; ci < S.child_ptr[J + 1]; ++ci) child = std::max(child, S.mJ[S.child_idx[ci]]);
+            const size_t sm = chf_smem((size_t)S.nJ[J] + S.mJ[J], S.nJ[J], child);
             c->lvl_factor_smem[h] = std::max(c->lvl_factor_smem[h], sm);
-            // factor block (rounded to 16 bytes), the vectors (rows of 12
-            // floats for up to 9 columns), the 128-row scratch, the node's
-            // FP64 solution entries, then the staged rows and update vectors
-            // of the children or struct(J) (see StepSmem)
-            size_t csum = 0;   // rows of the children's update vectors
-            for (int ci = S.child_ptr[J]; ci < S.child_ptr[J + 1]; ++ci) csum += S.mJ[S.child_idx[ci]];
-            const size_t ss = sizeof(float) * ((((size_t)S.nJ[J] * chol_ld(S.nJ[J]) +
-                                                 (size_t)S.nJ[J] * chol_ld(S.mJ[J]) + 3) & ~size_t(3)) +
-                                               ((size_t)S.mJ[J] + 2 * S.nJ[J]) * 12 + 128 * 12 +
-                                               2 * (size_t)S.nJ[J] * CH_KMAX +
-                                               std::max(csum * (CH_KMAX + 1), (size_t)S.mJ[J]));
-            c->lvl_solve_smem[h] = std::max(c->lvl_solve_smem[h], ss);
             worst = std::max(worst, sm);
+            if (S.child_ptr[J + 1] - S.child_ptr[J] == 1 && S.mJ[S.child_idx[S.child_ptr[J]]] == S.nJ[J] + S.mJ[J])
+                flags[J] |= CHN_INPLACE;
+            // a chain's link reads one vector in order, and a front whose children
+            // do not fit beside it reads theirs from global memory
+            if ((flags[J] & CHN_INPLACE) || step_smem(J, CH_KMAX, false) > CH_SMEM_MAX) flags[J] |= CHN_DIRECT;
+            for (int K = 1; K <= CH_KMAX; ++K)
+                lvl_smem[K] = std::max(lvl_smem[K], step_smem(J, K, flags[J] & CHN_DIRECT));
             // partial Cholesky, Schur update of struct x struct, triangular inverse
             c->lvl_factor_flops[h] += n * n * n / 3.0 + n * n * mm + n * mm * mm + n * n * n / 3.0;
         }
+        for (int K = 1; K <= CH_KMAX; ++K) {
+            c->solve_smem[K] = std::max(c->solve_smem[K], lvl_smem[K]);
+            small_open[K] = small_open[K] && lvl_smem[K] <= CHS_SMALL;
+            if (!small_open[K]) continue;
+            c->small_smem[K] = std::max(c->small_smem[K], lvl_smem[K]);
+            c->small_n[K] = S.level_ptr[h + 1];
+        }
+    }
     c->solve_bytes = 2.0 * sizeof(float) * (double)S.lsize;
-    size_t solve_smem = 0;
-    for (int h = 0; h < c->H; ++h) solve_smem = std::max(solve_smem, c->lvl_solve_smem[h]);
-    c->solve_smem = solve_smem;
-    if (worst > CH_SMEM_MAX || solve_smem > CH_SMEM_MAX) {
+    worst = std::max(worst, c->solve_smem[CH_KMAX]);
+    if (worst > CH_SMEM_MAX) {
         c->why = "a supernode panel needs " + std::to_string(worst) + " bytes of shared memory";
         m->chol = c.release();
         return TP_OK;
+    }
+    // update matrices: in place ones are the trailing part of the child's
+    std::vector<int64_t> uoff(S.nnode);
+    std::vector<int> ldu(S.nnode);
+    int64_t usize = 0;
+    for (int J = 0; J < S.nnode; ++J) {   // postorder: children first
+        if (flags[J] & CHN_INPLACE) {
+            const int ch = S.child_idx[S.child_ptr[J]];
+            ldu[J] = ldu[ch];
+            uoff[J] = uoff[ch] + (int64_t)S.nJ[J] * (ldu[ch] + 1);
+        } else {
+            ldu[J] = S.mJ[J];
+            uoff[J] = usize;
+            usize += (int64_t)S.mJ[J] * S.mJ[J];
+        }
+    }
+    // tiles of the update matrices (lower part), by level
+    std::vector<int4> tiles;
+    c->lvl_tile.assign(c->H + 1, 0);
+    for (int h = 0; h < c->H; ++h) {
+        for (int i = S.level_ptr[h]; i < S.level_ptr[h + 1]; ++i) {
+            const int J = S.level_nodes[i];
+            for (int c0 = 0; c0 < S.mJ[J]; c0 += CHF_TILE)
+                for (int r0 = c0; r0 < S.mJ[J]; r0 += CHF_TILE) tiles.push_back(make_int4(J, r0, c0, 0));
+        }
+        c->lvl_tile[h + 1] = (int)tiles.size();
     }
     // device tables
     std::vector<CholNode> nodes(S.nnode);
@@ -972,14 +1307,15 @@ static int chol_setup(tp_mesh* m) {
         d.mJ = S.mJ[J];
         d.t = S.nJ[J] + S.mJ[J];
         d.loff = S.loff[J];
-        d.uoff = S.uoff[J];
+        d.uoff = uoff[J];
         d.voff = S.voff[J];
         d.child0 = S.child_ptr[J];
         d.child1 = S.child_ptr[J + 1];
         d.s0 = S.struct_ptr[J];
         d.asm0 = S.asm_ptr[J];
         d.asm1 = S.asm_ptr[J + 1];
-        d.pad0 = d.pad1 = 0;
+        d.ldu = ldu[J];
+        d.flags = flags[J];
     }
     std::vector<int> comp_ptr(S.ncomp + 1, 0), comp_verts(nv);
     for (int v = 0; v < nv; ++v) comp_ptr[S.comp[v] + 1]++;
@@ -1000,21 +1336,22 @@ static int chol_setup(tp_mesh* m) {
     TP_TRY(upload(c->comp_verts, comp_verts));
     TP_TRY(upload(c->comp_of, S.comp));
     TP_TRY(upload(c->parent, S.parent));
+    TP_TRY(upload(c->tiles, tiles));
     TP_TRY(ensure(c->fdone, sizeof(unsigned) * std::max(1, S.nnode)));
     TP_TRY(ensure(c->bdone, sizeof(unsigned) * std::max(1, S.nnode)));
     TP_CUDA(cudaMemset(c->fdone.ptr, 0, sizeof(unsigned) * std::max(1, S.nnode)));
     TP_CUDA(cudaMemset(c->bdone.ptr, 0, sizeof(unsigned) * std::max(1, S.nnode)));
     TP_TRY(ensure(c->L, sizeof(float) * std::max<int64_t>(1, S.lsize)));
-    TP_TRY(ensure(c->U, sizeof(float) * std::max<int64_t>(1, S.usize)));
+    TP_TRY(ensure(c->U, sizeof(float) * std::max<int64_t>(1, usize)));
     TP_TRY(ensure(c->uvec, sizeof(float) * (size_t)std::max(1, S.vsize) * CH_KMAX));
     TP_TRY(ensure(c->ybuf, sizeof(float) * (size_t)std::max(1, S.n) * CH_KMAX));
     TP_TRY(ensure(c->xbuf, sizeof(float) * (size_t)std::max(1, S.n) * CH_KMAX));
     TP_TRY(ensure(c->ctl, sizeof(CholCtl)));
     TP_CUDA(cudaMemset(c->ctl.ptr, 0, sizeof(CholCtl)));
 #ifdef TP_CHOL_TRACE
-    TP_TRY(ensure(c->trace, sizeof(unsigned long long) * 6 * ((size_t)2 * S.nnode + 2 * sm_count() + 2)));
+    TP_TRY(ensure(c->trace, sizeof(unsigned long long) * 6 * ((size_t)2 * S.nnode + 3 * sm_count() + 2)));
 #endif
-    TP_CUDA(cudaFuncSetAttribute(k_chol_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CH_SMEM_MAX));
+    TP_CUDA(cudaFuncSetAttribute(k_chol_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CH_SMEM_MAX));
     TP_TRY(solve_smem_attr<1>());
     c->ok = true;
     m->chol = c.release();
@@ -1033,10 +1370,19 @@ static int chol_factor(tp_mesh* m, cudaStream_t st) {
         for (int h = 0; h < c->H; ++h) {
             const int cnt = S.level_ptr[h + 1] - S.level_ptr[h];
             if (cnt == 0) continue;
-            k_chol_factor<<<cnt, CHF_T, c->lvl_factor_smem[h], st>>>(
+            // small fronts by the thousand: more blocks per SM; above them the level
+            // waits for its largest front
+            const int threads = c->lvl_max_t[h] <= 96 ? 128 : cnt >= sm_count() ? 256 : 512;
+            k_chol_panel<<<cnt, threads, c->lvl_factor_smem[h], st>>>(
                 c->nodes.as<CholNode>(), c->level_nodes.as<int>() + S.level_ptr[h], c->child_idx.as<int>(),
                 c->rel.as<int>(), c->asm_dst.as<int>(), c->asm_src.as<int>(), m->val.as<double>(),
                 c->L.as<float>(), c->U.as<float>(), c->ctl.as<CholCtl>());
+            TP_LAUNCH_CHECK();
+            const int nt = c->lvl_tile[h + 1] - c->lvl_tile[h];
+            if (nt == 0) continue;
+            k_chol_update<<<nt, 256, 0, st>>>(c->nodes.as<CholNode>(), c->tiles.as<int4>() + c->lvl_tile[h],
+                                              c->child_idx.as<int>(), c->rel.as<int>(), c->L.as<float>(),
+                                              c->U.as<float>());
             TP_LAUNCH_CHECK();
         }
     }
@@ -1107,11 +1453,28 @@ static int chol_sweep_kernels(tp_mesh* m, int nsweep, int rgrid, double* partr, 
     A.nn = S.nnode;
     A.cap = cap;
     (void)rgrid;
-    const int grid = std::max(1, std::min(S.nnode, 2 * sm_count()));
+    const int nn = S.nnode, sms = sm_count(), small = c->small_n[K];
+    // One launch a sweep, with the shared memory of its largest step. Where that
+    // leaves one or two blocks per SM to thousands of small steps (163,842 vertices:
+    // 5,600 of 5,811), the small levels at the leaves run in launches of their own,
+    // forward before and backward after the others, three blocks per SM.
+    const bool parts = c->solve_smem[K] > CHS_SMALL && small >= 6 * sms;
     for (int s = 0; s < nsweep; ++s) {
-        k_chol_sweep<K><<<grid, CHS_T, c->solve_smem, st>>>(A);
-        TP_CUDA(cudaGetLastError());
-        ++*nk;
+        for (int part = 0; part < 3; ++part) {
+            if (!parts && part != 2) continue;
+            A.phase = part;
+            A.t0 = !parts || part == 0 ? 0 : part == 1 ? small : 2 * nn - small;
+            A.t1 = parts && part == 0 ? small : parts && part == 1 ? 2 * nn - small : 2 * nn;
+            A.last = part == 2;
+            const bool big = !parts || part == 1;
+            const int most = big ? 2 * sms : 3 * sms;
+            const int want = !parts ? nn : part == 1 ? nn - small : small;
+            const int grid = std::max(1, std::min(want, most));
+            if (want == 0) continue;
+            k_chol_sweep<K><<<grid, CHS_T, big ? c->solve_smem[K] : c->small_smem[K], st>>>(A);
+            TP_CUDA(cudaGetLastError());
+            ++*nk;
+        }
     }
     return TP_OK;
 }
@@ -1181,8 +1544,8 @@ static int chol_run(tp_mesh* m, const tp_params* p, const double* b, double* z_o
     const int rgrid = std::min(4 * sm_count(), (nv + CHR_T - 1) / CHR_T);
     // partial sums after the per-component means (comp_project's region)
     // per-block partials of the initial residual (rgrid blocks) and of the
-    // sweep kernel (up to 2 blocks per SM)
-    const size_t nparts = (size_t)std::max(rgrid, 2 * sm_count());
+    // sweep kernel (up to 3 blocks per SM)
+    const size_t nparts = (size_t)std::max(rgrid, 3 * sm_count());
     const size_t head = (size_t)c->ncomp * CH_KMAX * (1 + CH_MSPLIT);   // means and their slices
     TP_TRY(ensure(c->part, sizeof(double) * (head + nparts * CH_KMAX) + 64));
     double* partr = c->part.as<double>() + head;
@@ -1211,8 +1574,11 @@ static int chol_run(tp_mesh* m, const tp_params* p, const double* b, double* z_o
             TP_TRY(ensure(c->dflags, 4 * sizeof(int)));
             TP_CUDA(cudaMemsetAsync(c->dflags.ptr, 0, 4 * sizeof(int), st));   // fresh memory holds garbage
         }
+        // Larger meshes: 2.5 and 1.5 (163,842 vertices: 1e-4 in two sweeps, 1e-9 in
+        // four; 655,362: 1e-4 in three, 1e-6 in four).
         const double digits = -std::log10(std::max(p->cg_tol, 1e-300));
-        const int sweeps = std::min(cap, 1 + std::max(0, (int)std::ceil((digits - 4.0) / 3.0)));
+        const double first = nv <= 120000 ? 4.0 : 2.5, next = nv <= 120000 ? 3.0 : 1.5;
+        const int sweeps = std::min(cap, 1 + std::max(0, (int)std::ceil((digits - first) / next)));
         const int graphs = sweeps / CH_SWEEPS_PER_GRAPH;
         for (int gi = 0; gi < graphs; ++gi) {
             ProfScope ps(m, PK_CHOL_SOLVE, c->solve_bytes * CH_SWEEPS_PER_GRAPH, st);
