@@ -137,49 +137,14 @@ static NodeArrays node_arrays(const tp_mesh* m) {
 // device: Morton codes, sort, face boxes, node aggregates
 // ---------------------------------------------------------------------------
 
-__global__ void k_bbox_partial(const d4* __restrict__ X, int nf, double* __restrict__ part) {
-    __shared__ double lo[3][256], hi[3][256];
-    double l[3] = {1e300, 1e300, 1e300}, h[3] = {-1e300, -1e300, -1e300};
-    for (int i = blockIdx.x * 256 + threadIdx.x; i < nf; i += gridDim.x * 256) {
-        d4 x = X[i];
-        double v[3] = {x.x, x.y, x.z};
-        for (int c = 0; c < 3; ++c) {
-            l[c] = fmin(l[c], v[c]);
-            h[c] = fmax(h[c], v[c]);
-        }
-    }
-    for (int c = 0; c < 3; ++c) {
-        lo[c][threadIdx.x] = l[c];
-        hi[c][threadIdx.x] = h[c];
-    }
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int c = 0; c < 3; ++c) {
-                lo[c][threadIdx.x] = fmin(lo[c][threadIdx.x], lo[c][threadIdx.x + w]);
-                hi[c][threadIdx.x] = fmax(hi[c][threadIdx.x], hi[c][threadIdx.x + w]);
-            }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0)
-        for (int c = 0; c < 3; ++c) {
-            part[6 * blockIdx.x + c] = lo[c][0];
-            part[6 * blockIdx.x + 3 + c] = hi[c][0];
-        }
-}
-
-__global__ void k_bbox_final(double* __restrict__ part, int nblk) {
-    if (threadIdx.x != 0) return;
-    double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
-    for (int b = 0; b < nblk; ++b)
-        for (int c = 0; c < 3; ++c) {
-            lo[c] = fmin(lo[c], part[6 * b + c]);
-            hi[c] = fmax(hi[c], part[6 * b + 3 + c]);
-        }
-    for (int c = 0; c < 3; ++c) {
-        part[6 * 1024 + c] = lo[c];
-        part[6 * 1024 + 3 + c] = hi[c];
-    }
+// bounding box of the barycenters: bb = {lo, hi}
+__global__ void __launch_bounds__(256)
+k_bary_bbox(const d4* __restrict__ X, int nf, double* __restrict__ part, unsigned* __restrict__ ticket,
+            double* __restrict__ bb) {
+    bbox_points([&](int i, double* v) { const d4 x = X[i]; v[0] = x.x; v[1] = x.y; v[2] = x.z; }, nf, part, ticket,
+                [&](const double* lo, const double* hi) {
+                    for (int c = 0; c < 3; ++c) bb[c] = lo[c], bb[3 + c] = hi[c];
+                });
 }
 
 __device__ __forceinline__ unsigned spread10(unsigned v) {
@@ -408,10 +373,10 @@ int bvh_build(tp_mesh* m, const tp_params* p, cudaStream_t st) {
         k_keys_from_perm<<<(nf + 255) / 256, 256, 0, st>>>(perm, nf, kout);
         TP_LAUNCH_CHECK();
     } else {
-        int nblk = std::min(1024, (nf + 255) / 256);
-        k_bbox_partial<<<nblk, 256, 0, st>>>(m->f64a.as<d4>(), nf, bpart);
-        TP_LAUNCH_CHECK();
-        k_bbox_final<<<1, 32, 0, st>>>(bpart, nblk);
+        const int nblk = std::max(1, std::min(2 * sm_count(), (nf + 1023) / 1024));
+        unsigned* tk = nullptr;
+        TP_TRY(mesh_tickets(m, &tk, st));
+        k_bary_bbox<<<nblk, 256, 0, st>>>(m->f64a.as<d4>(), nf, bpart, tk + TICKET_BBOX, bpart + 6 * 1024);
         TP_LAUNCH_CHECK();
         k_morton<<<(nf + 255) / 256, 256, 0, st>>>(m->f64a.as<d4>(), nf, bpart + 6 * 1024, kin);
         TP_LAUNCH_CHECK();

@@ -1,5 +1,6 @@
 // Mesh state: face geometry (X_S, N_S, a_S and hat gradients), the
 // face-corner -> vertex gather, copies and deterministic FP64 sums.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -230,101 +231,108 @@ int sum_f64(const double* x, int n, double* out_dev, tp_mesh* m, cudaStream_t st
 // face geometry, §3.1 / §3.2.1
 // ---------------------------------------------------------------------------
 
-__global__ void k_face_geom(const double* __restrict__ pos, const int* __restrict__ faces, int nf,
-                            const double* __restrict__ center, float4* __restrict__ f32a,
-                            float4* __restrict__ f32b, float4* __restrict__ f32c, d4* __restrict__ f64a,
-                            d4* __restrict__ f64b, double* __restrict__ fgrad, int* __restrict__ err) {
-    int S = blockIdx.x * blockDim.x + threadIdx.x;
-    if (S >= nf) return;
-    int i = faces[3 * S], j = faces[3 * S + 1], k = faces[3 * S + 2];
-    double pi[3], pj[3], pk[3];
-    for (int c = 0; c < 3; ++c) {
-        pi[c] = pos[3 * i + c];
-        pj[c] = pos[3 * j + c];
-        pk[c] = pos[3 * k + c];
-    }
-    double e1[3] = {pj[0] - pi[0], pj[1] - pi[1], pj[2] - pi[2]};
-    double e2[3] = {pk[0] - pi[0], pk[1] - pi[1], pk[2] - pi[2]};
-    double n[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2],
-                   e1[0] * e2[1] - e1[1] * e2[0]};
-    double nn = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-    bool ok = nn > 0.0 && isfinite(nn);
-    for (int c = 0; c < 3; ++c) ok = ok && isfinite(pi[c]) && isfinite(pj[c]) && isfinite(pk[c]);
-    if (!ok) {
-        atomicOr(err, 1);
-        nn = 1.0;
-    }
-    double a = 0.5 * nn;
-    double N[3] = {n[0] / nn, n[1] / nn, n[2] / nn};
-    double X[3];
-    for (int c = 0; c < 3; ++c) X[c] = (pi[c] + pj[c] + pk[c]) / 3.0 - center[c];
-    f64a[S] = d4{X[0], X[1], X[2], a};
-    f64b[S] = d4{N[0], N[1], N[2], 0.0};
-    f32a[S] = make_float4((float)X[0], (float)X[1], (float)X[2], (float)a);
-    f32c[S] = make_float4((float)(X[0] - (double)(float)X[0]), (float)(X[1] - (double)(float)X[1]),
-                          (float)(X[2] - (double)(float)X[2]), 0.0f);
-    f32b[S] = make_float4((float)N[0], (float)N[1], (float)N[2], 0.0f);
-    // hat gradients: grad phi_c = N x e_c / (2a), e_c the edge opposite corner c
-    const double* P[3] = {pi, pj, pk};
-    for (int c = 0; c < 3; ++c) {
-        const double* p1 = P[(c + 1) % 3];
-        const double* p2 = P[(c + 2) % 3];
-        double e[3] = {p2[0] - p1[0], p2[1] - p1[1], p2[2] - p1[2]};
-        double g[3] = {N[1] * e[2] - N[2] * e[1], N[2] * e[0] - N[0] * e[2],
-                       N[0] * e[1] - N[1] * e[0]};
-        for (int q = 0; q < 3; ++q) fgrad[9 * S + 3 * c + q] = g[q] / (2.0 * a);
-    }
-}
-
-// bounding box of the vertices: per-block min/max, then the centre (lo+hi)/2
-__global__ void k_pos_bbox_partial(const double* __restrict__ pos, int nv, double* __restrict__ part) {
-    __shared__ double lo[3][256], hi[3][256];
-    double l[3] = {1e300, 1e300, 1e300}, h[3] = {-1e300, -1e300, -1e300};
-    for (int i = blockIdx.x * 256 + threadIdx.x; i < nv; i += gridDim.x * 256)
+// One thread per face, a block per tile of 128 consecutive faces, whose box of FP32
+// barycenters (source tiles of the pair kernels) it leaves too. Bound by the FP64
+// pipe on large meshes: 120 operations a face (250 with the compiler's divisions and
+// square root: 132 us on 327,680 faces, now 88 us), by latency on small ones.
+__global__ void __launch_bounds__(128)
+k_face_geom(const double* __restrict__ pos, const int* __restrict__ faces, int nf,
+            const double* __restrict__ center, float4* __restrict__ f32a, float4* __restrict__ f32b,
+            float4* __restrict__ f32c, d4* __restrict__ f64a, d4* __restrict__ f64b, double* __restrict__ fgrad,
+            float4* __restrict__ box, int* __restrict__ err) {
+    const int S = blockIdx.x * 128 + threadIdx.x, lane = threadIdx.x & 31;
+    float lo[3] = {3e38f, 3e38f, 3e38f}, hi[3] = {-3e38f, -3e38f, -3e38f};
+    if (S < nf) {
+        const int i = faces[3 * S], j = faces[3 * S + 1], k = faces[3 * S + 2];
+        double pi[3], pj[3], pk[3];
         for (int c = 0; c < 3; ++c) {
-            l[c] = fmin(l[c], pos[3 * i + c]);
-            h[c] = fmax(h[c], pos[3 * i + c]);
+            pi[c] = pos[3 * (size_t)i + c];
+            pj[c] = pos[3 * (size_t)j + c];
+            pk[c] = pos[3 * (size_t)k + c];
         }
-    for (int c = 0; c < 3; ++c) {
-        lo[c][threadIdx.x] = l[c];
-        hi[c][threadIdx.x] = h[c];
+        const double e1[3] = {pj[0] - pi[0], pj[1] - pi[1], pj[2] - pi[2]};
+        const double e2[3] = {pk[0] - pi[0], pk[1] - pi[1], pk[2] - pi[2]};
+        const double n[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2],
+                             e1[0] * e2[1] - e1[1] * e2[0]};
+        double rn;
+        double nn = sqrt64(n[0] * n[0] + n[1] * n[1] + n[2] * n[2], &rn);
+        bool ok = nn > 0.0 && isfinite(nn);
+        for (int c = 0; c < 3; ++c) ok = ok && isfinite(pi[c]) && isfinite(pj[c]) && isfinite(pk[c]);
+        if (!ok) {
+            atomicOr(err, 1);
+            nn = rn = 1.0;
+        }
+        const double a = 0.5 * nn;
+        const double N[3] = {div64(n[0], nn, rn), div64(n[1], nn, rn), div64(n[2], nn, rn)};
+        double X[3];
+        float Xf[3];
+        for (int c = 0; c < 3; ++c) {
+            X[c] = third64(pi[c] + pj[c] + pk[c]) - center[c];
+            Xf[c] = (float)X[c];
+            lo[c] = hi[c] = Xf[c];
+        }
+        f64a[S] = d4{X[0], X[1], X[2], a};
+        f64b[S] = d4{N[0], N[1], N[2], 0.0};
+        f32a[S] = make_float4(Xf[0], Xf[1], Xf[2], (float)a);
+        f32c[S] = make_float4((float)(X[0] - (double)Xf[0]), (float)(X[1] - (double)Xf[1]),
+                              (float)(X[2] - (double)Xf[2]), 0.0f);
+        f32b[S] = make_float4((float)N[0], (float)N[1], (float)N[2], 0.0f);
+        // hat gradients: grad phi_c = N x e_c / (2a), e_c the edge opposite corner c
+        // (e_1 = -e2 and e_2 = e1 of above)
+        const double e0[3] = {pk[0] - pj[0], pk[1] - pj[1], pk[2] - pj[2]};
+        for (int c = 0; c < 3; ++c) {
+            const double* e = c == 0 ? e0 : c == 1 ? e2 : e1;
+            const double sg = c == 1 ? -1.0 : 1.0;
+            const double g[3] = {N[1] * e[2] - N[2] * e[1], N[2] * e[0] - N[0] * e[2], N[0] * e[1] - N[1] * e[0]};
+            for (int q = 0; q < 3; ++q) fgrad[9 * (size_t)S + 3 * c + q] = sg * div64(g[q], nn, rn);
+        }
     }
+    __shared__ float sb[4][6];
+    for (int o = 16; o > 0; o >>= 1)
+        for (int c = 0; c < 3; ++c) {
+            lo[c] = fminf(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
+            hi[c] = fmaxf(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
+        }
+    if (lane == 0)
+        for (int c = 0; c < 3; ++c) {
+            sb[threadIdx.x >> 5][c] = lo[c];
+            sb[threadIdx.x >> 5][3 + c] = hi[c];
+        }
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 4; ++w)
             for (int c = 0; c < 3; ++c) {
-                lo[c][threadIdx.x] = fmin(lo[c][threadIdx.x], lo[c][threadIdx.x + w]);
-                hi[c][threadIdx.x] = fmax(hi[c][threadIdx.x], hi[c][threadIdx.x + w]);
+                lo[c] = fminf(lo[c], sb[w][c]);
+                hi[c] = fmaxf(hi[c], sb[w][3 + c]);
             }
-        __syncthreads();
+        box[2 * blockIdx.x] = make_float4(lo[0], lo[1], lo[2], 0.f);
+        box[2 * blockIdx.x + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
     }
-    if (threadIdx.x == 0)
-        for (int c = 0; c < 3; ++c) {
-            part[6 * blockIdx.x + c] = lo[c][0];
-            part[6 * blockIdx.x + 3 + c] = hi[c][0];
-        }
 }
 
-__global__ void k_pos_bbox_center(const double* __restrict__ part, int nblk, double* __restrict__ center) {
-    if (threadIdx.x != 0) return;
-    double half[3];
-    for (int c = 0; c < 3; ++c) {
-        double l = 1e300, h = -1e300;
-        for (int b = 0; b < nblk; ++b) {
-            l = fmin(l, part[6 * b + c]);
-            h = fmax(h, part[6 * b + 3 + c]);
-        }
-        center[c] = 0.5 * (l + h);
-        half[c] = 0.5 * (h - l);
-    }
-    // source tiles closer than R/16 to a target block (R = half diagonal of
-    // the bounding box) take the compensated barycenter difference: beyond
-    // it the FP32 rounding of the barycenters perturbs |d| by < 2^-19
-    double R2 = half[0] * half[0] + half[1] * half[1] + half[2] * half[2];
-    center[3] = R2 / 256.0;
+// bounding box of the vertices: the centre (lo+hi)/2 is the frame of the face
+// tables; the geometry's error flag starts at zero
+__global__ void __launch_bounds__(256)
+k_pos_bbox(const double* __restrict__ pos, int nv, double* __restrict__ part, unsigned* __restrict__ ticket,
+           double* __restrict__ center, int* __restrict__ err) {
+    bbox_points([&](int i, double* v) { for (int c = 0; c < 3; ++c) v[c] = pos[3 * (size_t)i + c]; }, nv, part, ticket,
+                [&](const double* lo, const double* hi) {
+                    double R2 = 0.0;
+                    for (int c = 0; c < 3; ++c) {
+                        center[c] = 0.5 * (lo[c] + hi[c]);
+                        const double half = 0.5 * (hi[c] - lo[c]);
+                        R2 += half * half;
+                    }
+                    // source tiles closer than R/16 to a target block (R = half diagonal of
+                    // the bounding box) take the compensated barycenter difference: beyond
+                    // it the FP32 rounding of the barycenters perturbs |d| by < 2^-19
+                    center[3] = R2 / 256.0;
+                    for (int c = 0; c < 4; ++c) err[c] = 0;
+                });
 }
 
-// bounding box of the FP32 barycenters of each tile of 128 consecutive faces
+// bounding box of the FP32 barycenters of each tile of 128 consecutive faces (of an
+// obstacle in the surface's frame; k_face_geom does its own)
 __global__ void k_tile_boxes(const float4* __restrict__ f32a, int nf, float4* __restrict__ box) {
     __shared__ float lo[3][128], hi[3][128];
     int S = blockIdx.x * 128 + threadIdx.x;
@@ -405,28 +413,20 @@ int project_components(tp_mesh* m, double* x, int k, cudaStream_t st) {
 int refresh_geometry(tp_mesh* m, cudaStream_t st) {
     // reference frame: centre of the vertices' bounding box (exact in FP64),
     // so that the FP32 face table holds barycenters relative to the mesh
-    {
-        int nblk = (m->nv + 255) / 256;
-        if (nblk > 256) nblk = 256;
-        TP_TRY(ensure(m->part2, sizeof(double) * 6 * (size_t)nblk));
-        k_pos_bbox_partial<<<nblk, 256, 0, st>>>(m->pos.as<double>(), m->nv, m->part2.as<double>());
-        TP_LAUNCH_CHECK();
-        k_pos_bbox_center<<<1, 32, 0, st>>>(m->part2.as<double>(), nblk, m->center.as<double>());
-        TP_LAUNCH_CHECK();
-    }
-    TP_CUDA(cudaMemsetAsync(m->errflag.ptr, 0, sizeof(int) * 4, st));
-    int nb = (m->nf + 255) / 256;
-    k_face_geom<<<nb, 256, 0, st>>>(m->pos.as<double>(), m->faces.as<int>(), m->nf,
-                                    m->center.as<double>(), m->f32a.as<float4>(),
-                                    m->f32b.as<float4>(), m->f32c.as<float4>(), m->f64a.as<d4>(),
-                                    m->f64b.as<d4>(), m->fgrad.as<double>(), m->errflag.as<int>());
+    const int nblk = std::max(1, std::min(2 * sm_count(), (m->nv + 1023) / 1024));
+    const int ntiles = (m->nf + 127) / 128;
+    unsigned* tk = nullptr;
+    TP_TRY(mesh_tickets(m, &tk, st));
+    TP_TRY(ensure(m->part2, sizeof(double) * 6 * (size_t)nblk));
+    TP_TRY(ensure(m->tilebox, sizeof(float4) * 2 * (size_t)ntiles));
+    k_pos_bbox<<<nblk, 256, 0, st>>>(m->pos.as<double>(), m->nv, m->part2.as<double>(), tk + TICKET_BBOX,
+                                     m->center.as<double>(), m->errflag.as<int>());
     TP_LAUNCH_CHECK();
-    {
-        int ntiles = (m->nf + 127) / 128;
-        TP_TRY(ensure(m->tilebox, sizeof(float4) * 2 * (size_t)ntiles));
-        k_tile_boxes<<<ntiles, 128, 0, st>>>(m->f32a.as<float4>(), m->nf, m->tilebox.as<float4>());
-        TP_LAUNCH_CHECK();
-    }
+    k_face_geom<<<ntiles, 128, 0, st>>>(m->pos.as<double>(), m->faces.as<int>(), m->nf, m->center.as<double>(),
+                                        m->f32a.as<float4>(), m->f32b.as<float4>(), m->f32c.as<float4>(),
+                                        m->f64a.as<d4>(), m->f64b.as<d4>(), m->fgrad.as<double>(),
+                                        m->tilebox.as<float4>(), m->errflag.as<int>());
+    TP_LAUNCH_CHECK();
     TP_TRY(obstacle_frame(m, st));   // the frame moved with the positions
     int err = 0;
     TP_CUDA(cudaMemcpyAsync(&err, m->errflag.ptr, sizeof(int), cudaMemcpyDeviceToHost, st));

@@ -71,6 +71,108 @@ struct alignas(32) d4 {
 int sm_count();
 
 // ---------------------------------------------------------------------------
+// FP64 divisions and roots in few operations
+// ---------------------------------------------------------------------------
+//
+// The FP64 pipe issues two lanes a cycle and SM, and the compiler's division and
+// square root are sequences of 10 to 20 operations on it. These start from the
+// 20-bit approximations and take one third-order step; a quotient or root then gets
+// a residual correction, which makes it the correctly rounded one but for rare ties.
+
+// reciprocal of a normal x
+__device__ __forceinline__ double rcp64(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+// a / b with r = 1 / b (to about an ulp)
+__device__ __forceinline__ double div64(double a, double b, double r) {
+    const double q = a * r;
+    return fma(fma(-q, b, a), r, q);
+}
+// sqrt(x), and its reciprocal in *r; x outside [1e-280, 1e280] takes the functions
+__device__ __forceinline__ double sqrt64(double x, double* r) {
+    if (!(x > 1e-280 && x < 1e280)) {
+        const double s = sqrt(x);
+        *r = 1.0 / s;
+        return s;
+    }
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x * y, y, 1.0);
+    y = fma(y * e, fma(e, 0.375, 0.5), y);
+    const double s0 = x * y;
+    const double s = fma(fma(-s0, s0, x), 0.5 * y, s0);
+    *r = fma(y, fma(-s, y, 1.0), y);
+    return s;
+}
+__device__ __forceinline__ double third64(double x) { return div64(x, 3.0, 1.0 / 3.0); }
+
+// ---------------------------------------------------------------------------
+// bounding box of points in one launch
+// ---------------------------------------------------------------------------
+//
+// part [6 gridDim] and the completion ticket (zero between launches): each block's
+// box, then the last block to finish takes the box of those (minima and maxima, so
+// the order does not matter). done(lo, hi) runs in one thread of the last block.
+// With the blocks' boxes left to one thread of a second launch this took 105 us on
+// 163,842 vertices and 412 us on 327,680 faces.
+template <class Load, class Done>
+__device__ __forceinline__ void bbox_points(Load load, int n, double* part, unsigned* ticket, Done done) {
+    __shared__ double sh[8][6];
+    __shared__ bool last;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;   // 256 threads
+    double b[6] = {1e300, 1e300, 1e300, -1e300, -1e300, -1e300};
+    auto fold = [&]() {   // of the block, in thread 0
+        for (int o = 16; o > 0; o >>= 1)
+            for (int c = 0; c < 3; ++c) {
+                b[c] = fmin(b[c], __shfl_xor_sync(0xffffffffu, b[c], o));
+                b[3 + c] = fmax(b[3 + c], __shfl_xor_sync(0xffffffffu, b[3 + c], o));
+            }
+        if (lane == 0)
+            for (int c = 0; c < 6; ++c) sh[w][c] = b[c];
+        __syncthreads();
+        if (tid == 0)
+            for (int q = 1; q < 8; ++q)
+                for (int c = 0; c < 3; ++c) {
+                    b[c] = fmin(b[c], sh[q][c]);
+                    b[3 + c] = fmax(b[3 + c], sh[q][3 + c]);
+                }
+    };
+    for (int i = blockIdx.x * 256 + tid; i < n; i += gridDim.x * 256) {
+        double v[3];
+        load(i, v);
+        for (int c = 0; c < 3; ++c) {
+            b[c] = fmin(b[c], v[c]);
+            b[3 + c] = fmax(b[3 + c], v[c]);
+        }
+    }
+    fold();
+    if (gridDim.x > 1) {
+        if (tid == 0) {
+            for (int c = 0; c < 6; ++c) part[6 * blockIdx.x + c] = b[c];
+            __threadfence();
+            last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        }
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        for (int c = 0; c < 3; ++c) b[c] = 1e300, b[3 + c] = -1e300;
+        for (int q = tid; q < gridDim.x; q += 256)
+            for (int c = 0; c < 3; ++c) {
+                b[c] = fmin(b[c], __ldcg(part + 6 * q + c));
+                b[3 + c] = fmax(b[3 + c], __ldcg(part + 6 * q + 3 + c));
+            }
+        fold();
+    }
+    if (tid == 0) {
+        done(b, b + 3);
+        *ticket = 0u;
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Barnes-Hut tree (implicit, Morton-ordered; built on the device)
 // ---------------------------------------------------------------------------
 
@@ -293,7 +395,7 @@ int sum_f64(const double* x, int n, double* out_dev, tp_mesh* m, cudaStream_t st
 int colsum(tp_mesh* m, const double* x, long n, int k, double scale, double* out_dev, cudaStream_t st);
 // completion tickets of the fused (single-launch) reductions: one slot per
 // reduction kind, zero between launches
-enum { TICKET_COLSUM = 0, TICKET_DOTS = 1, TICKET_COMP = 2, TICKET_CHOL = 3, TICKET_COUNT = 8 };
+enum { TICKET_COLSUM = 0, TICKET_DOTS = 1, TICKET_COMP = 2, TICKET_CHOL = 3, TICKET_BBOX = 4, TICKET_ENERGY = 5, TICKET_COUNT = 8 };
 int mesh_tickets(tp_mesh* m, unsigned** out, cudaStream_t st);
 const char* last_error();
 // profiling: wrap a launch (or a group of launches) of kernel class `key`
