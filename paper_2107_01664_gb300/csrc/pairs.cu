@@ -612,36 +612,6 @@ __device__ __forceinline__ void diff_term(T dx, T dy, T dz, T nx, T ny, T nz, T 
     pt[11] += kS;
 }
 
-// diff_term (p = 6) for two targets (lanes) against one source, packed;
-// pt[i] holds accumulator i of both targets
-__device__ __forceinline__ void diff_pair_p6(float2 dx, float2 dy, float2 dz, float2 nx, float2 ny, float2 nz, float at,
-                                             float mx, float my, float mz, float2* pt) {
-    const float2 r2 = f2fma(dx, dx, f2fma(dy, dy, f2fma(dz, dz, f2b(tiny_r2<float>()))));
-    const float2 ir2 = make_float2(rcp_(r2.x), rcp_(r2.y));
-    const float2 tS = f2mul(f2fma(nx, dx, f2fma(ny, dy, f2mul(nz, dz))), ir2);
-    const float2 tT = f2mul(f2fma(f2b(mx), dx, f2fma(f2b(my), dy, f2mul(f2b(mz), dz))), ir2);
-    const float2 qS = f2mul(tS, tS), qT = f2mul(tT, tT);
-    const float2 mS = f2mul(qS, qS), mT = f2mul(qT, qT);
-    const float2 A = f2b(at);
-    const float2 w = f2mul(f2mul(A, mS), f2mul(tS, ir2));
-    const float2 v = f2mul(f2mul(A, mT), f2mul(tT, ir2));
-    const float2 kS = f2mul(A, f2mul(mS, qS));
-    const float2 ks = f2fma(A, f2mul(mT, qT), kS);
-    const float2 kd = f2mul(ks, ir2);
-    pt[0] = f2add(pt[0], w);
-    pt[1] = f2fma(w, dx, pt[1]);
-    pt[2] = f2fma(w, dy, pt[2]);
-    pt[3] = f2fma(w, dz, pt[3]);
-    pt[4] = f2fma(v, f2b(mx), pt[4]);
-    pt[5] = f2fma(v, f2b(my), pt[5]);
-    pt[6] = f2fma(v, f2b(mz), pt[6]);
-    pt[7] = f2fma(kd, dx, pt[7]);
-    pt[8] = f2fma(kd, dy, pt[8]);
-    pt[9] = f2fma(kd, dz, pt[9]);
-    pt[10] = f2add(pt[10], ks);
-    pt[11] = f2add(pt[11], kS);
-}
-
 template <typename T, bool P6, int TT>
 __global__ void __launch_bounds__(NT)
 k_diff(const typename V4T<T>::type* __restrict__ fa, const typename V4T<T>::type* __restrict__ fb,
@@ -713,27 +683,6 @@ k_diff(const typename V4T<T>::type* __restrict__ fa, const typename V4T<T>::type
                                          (tz[j] - s.z) + (T)(lz[j] - l.z), nx[j], ny[j], nz[j], s.w, n.x, n.y,
                                          n.z, hm1, pt[j]);
                 }
-            } else if constexpr (F32 && P6 && TT == 2) {
-                // both targets per packed instruction
-                float2 p2[NADJ];
-#pragma unroll
-                for (int i = 0; i < NADJ; ++i) p2[i] = make_float2(0.f, 0.f);
-                const float2 TXp = make_float2((float)tx[0], (float)tx[1]), TYp = make_float2((float)ty[0], (float)ty[1]),
-                             TZp = make_float2((float)tz[0], (float)tz[1]);
-                const float2 NXp = make_float2((float)nx[0], (float)nx[1]), NYp = make_float2((float)ny[0], (float)ny[1]),
-                             NZp = make_float2((float)nz[0], (float)nz[1]);
-#pragma unroll 4
-                for (int q = 0; q < CH; ++q) {
-                    const float4 s = reinterpret_cast<const float4&>(sa[c + q]);
-                    const float4 n = reinterpret_cast<const float4&>(sb[c + q]);
-                    diff_pair_p6(f2sub(TXp, f2b(s.x)), f2sub(TYp, f2b(s.y)), f2sub(TZp, f2b(s.z)), NXp, NYp, NZp, s.w,
-                                 n.x, n.y, n.z, p2);
-                }
-#pragma unroll
-                for (int i = 0; i < NADJ; ++i) {
-                    pt[0][i] = p2[i].x;
-                    pt[1][i] = p2[i].y;
-                }
             } else {
 #pragma unroll 4
                 for (int q = 0; q < CH; ++q) {
@@ -759,32 +708,40 @@ k_diff(const typename V4T<T>::type* __restrict__ fa, const typename V4T<T>::type
                 part[((size_t)blockIdx.y * NADJ + i) * nt + tid[j]] = acc[j][i].value();
 }
 
-// adj[S*7 + 0..2] = dE/dX_S, [3..5] = dE/dN_S, [6] = dE/da_S; erow[S] = energy row
-__global__ void k_diff_combine(const double* __restrict__ part, int nsplit, int nf, double p,
-                               const d4* __restrict__ f64a, const d4* __restrict__ f64b,
-                               double* __restrict__ adj, double* __restrict__ erow) {
-    int S = blockIdx.x * blockDim.x + threadIdx.x;
-    if (S >= nf) return;
-    double s[NADJ];
-    for (int i = 0; i < NADJ; ++i) s[i] = 0.0;
-    for (int k = 0; k < nsplit; ++k)
-        for (int i = 0; i < NADJ; ++i) s[i] += part[((size_t)k * NADJ + i) * nf + S];
-    double a = f64a[S].w;
-    d4 N = f64b[S];
-    double NS[3] = {N.x, N.y, N.z};
-    for (int c = 0; c < 3; ++c) {
-        adj[7 * S + c] = a * (p * (s[0] * NS[c] + s[4 + c]) - 2.0 * p * s[7 + c]);
-        adj[7 * S + 3 + c] = a * p * s[1 + c];
+// adj[S*7 + 0..2] = dE/dX_S, [3..5] = dE/dN_S, [6] = dE/da_S; erow[S] = energy row.
+// A block takes 32 faces, a thread per (face, sum); one thread per face walked all
+// sums of all splits alone (33 us on 20,000 faces and 23 splits, now 13 us).
+__global__ void __launch_bounds__(32 * NADJ)
+k_diff_combine(const double* __restrict__ part, int nsplit, int nf, double p, const d4* __restrict__ f64a,
+               const d4* __restrict__ f64b, double* __restrict__ adj, double* __restrict__ erow) {
+    __shared__ double s[NADJ][33];
+    const int fl = threadIdx.x, i = threadIdx.y, S = blockIdx.x * 32 + fl;
+    double x = 0.0;
+    if (S < nf) {
+        const double* ps = part + (size_t)i * nf + S;
+#pragma unroll 4
+        for (int k = 0; k < nsplit; ++k) x += ps[(size_t)k * NADJ * nf];
     }
-    adj[7 * S + 6] = s[10];
-    if (erow) erow[S] = a * s[11];
+    s[i][fl] = x;
+    __syncthreads();
+    if (S >= nf || i > 3) return;
+    const double a = f64a[S].w;
+    if (i == 3) {
+        adj[7 * (size_t)S + 6] = s[10][fl];
+        if (erow) erow[S] = a * s[11][fl];
+        return;
+    }
+    const d4 N = f64b[S];
+    const double n = i == 0 ? N.x : i == 1 ? N.y : N.z;
+    adj[7 * (size_t)S + i] = a * (p * (s[0][fl] * n + s[4 + i][fl]) - 2.0 * p * s[7 + i][fl]);
+    adj[7 * (size_t)S + 3 + i] = a * p * s[1 + i][fl];
 }
 
 template <typename T>
 static int launch_diff(tp_mesh* m, const tp_params* p, double* adj, double* erow, cudaStream_t st) {
     using V4 = typename V4T<T>::type;
     constexpr int TT = sizeof(T) == 4 ? 2 : 1;
-    Grid g = make_grid(m->nf, m->nf, TT, resident_per_sm((const void*)k_diff<T, true, TT>, NT));
+    Grid g = make_grid(m->nf, m->nf, TT, resident_per_sm((const void*)k_diff<T, false, TT>, NT));
     if (sizeof(T) == 8) g = fp64_grid(g, m->nf);
     TP_TRY(ensure(m->part, sizeof(double) * (size_t)g.nsplit * NADJ * m->nf));
     const V4* fa = (const V4*)(sizeof(T) == 4 ? m->f32a.ptr : m->f64a.ptr);
@@ -794,17 +751,22 @@ static int launch_diff(tp_mesh* m, const tp_params* p, double* adj, double* erow
     m->pairs += units;
     {
         ProfScope ps(m, PK_DIFF, units, st);
-        if (p->p == 6.0)
-            k_diff<T, true, TT><<<grid, NT, sizeof(T) == 8 ? two_resident(k_diff<T, true, TT>) : 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
-                                                     m->center.as<double>(), m->nf, g.tiles_per_split, T(2),
-                                                     m->part.as<double>());
-        else
-            k_diff<T, false, TT><<<grid, NT, sizeof(T) == 8 ? two_resident(k_diff<T, false, TT>) : 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
-                                                      m->center.as<double>(), m->nf, g.tiles_per_split,
-                                                      T(0.5 * p->p - 1.0), m->part.as<double>());
+        // (FP32 at p = 6 runs in energy.cu)
+        bool p6 = false;
+        if constexpr (sizeof(T) == 8) {
+            p6 = p->p == 6.0;
+            if (p6)
+                k_diff<T, true, TT><<<grid, NT, two_resident(k_diff<T, true, TT>), st>>>(
+                    fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(), m->center.as<double>(), m->nf,
+                    g.tiles_per_split, T(2), m->part.as<double>());
+        }
+        if (!p6)
+            k_diff<T, false, TT><<<grid, NT, sizeof(T) == 8 ? two_resident(k_diff<T, false, TT>) : 0, st>>>(
+                fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(), m->center.as<double>(), m->nf,
+                g.tiles_per_split, T(0.5 * p->p - 1.0), m->part.as<double>());
         TP_LAUNCH_CHECK();
     }
-    k_diff_combine<<<(m->nf + 255) / 256, 256, 0, st>>>(m->part.as<double>(), g.nsplit, m->nf,
+    k_diff_combine<<<(m->nf + 31) / 32, dim3(32, NADJ), 0, st>>>(m->part.as<double>(), g.nsplit, m->nf,
                                                         p->p, m->f64a.as<d4>(), m->f64b.as<d4>(),
                                                         adj, erow);
     TP_LAUNCH_CHECK();

@@ -17,44 +17,60 @@ namespace tp {
 // energy / differential dispatch
 // ---------------------------------------------------------------------------
 
+// rowsum: [0] E of the pair sums, [1] the Willmore energy, [2] the obstacle's energy
+// where it was not added to the rows of [0]
+static int read_energy(tp_mesh* m, bool wm, bool obs, double* E_host, cudaStream_t st) {
+    double r[3] = {0.0, 0.0, 0.0};
+    TP_CUDA(cudaMemcpyAsync(r, m->rowsum.ptr, sizeof(double) * (obs ? 3 : wm ? 2 : 1), cudaMemcpyDeviceToHost, st));
+    TP_CUDA(cudaStreamSynchronize(st));
+    *E_host = r[0] + (wm ? m->willmore_w * r[1] : 0.0) + (obs ? r[2] : 0.0);
+    return TP_OK;
+}
+
 int energy_value(tp_mesh* m, const tp_params* p, double* E_host, cudaStream_t st, bool aux) {
     TP_TRY(ensure(m->erow, sizeof(double) * m->nf));
     TP_TRY(ensure(m->rowsum, sizeof(double) * 8));
-    if (p->theta > 0.0)
+    double* sums = m->rowsum.as<double>();
+    const bool wm = aux && m->willmore_w > 0.0, total = p6_fp32_direct(p), obs = aux && m->obs && total;
+    if (total)
+        TP_TRY(energy_total_p6(m, sums, st));
+    else if (p->theta > 0.0)
         TP_TRY(energy_rows_bh(m, p, nullptr, m->nf, m->erow.as<double>(), st));
     else
         TP_TRY(energy_rows_direct(m, p, nullptr, m->nf, m->erow.as<double>(), st));
-    if (aux) TP_TRY(obstacle_terms(m, p, false, true, m->erow.as<double>(), nullptr, st));
-    TP_TRY(sum_f64(m->erow.as<double>(), m->nf, m->rowsum.as<double>(), m, st));
-    const bool wm = aux && m->willmore_w > 0.0;
-    if (wm) TP_TRY(willmore_eval(m, m->rowsum.as<double>() + 1, nullptr, 0.0, st));
-    double r[2] = {0.0, 0.0};
-    TP_CUDA(cudaMemcpyAsync(r, m->rowsum.ptr, sizeof(double) * (wm ? 2 : 1), cudaMemcpyDeviceToHost, st));
-    TP_CUDA(cudaStreamSynchronize(st));
-    *E_host = r[0] + (wm ? m->willmore_w * r[1] : 0.0);
-    return TP_OK;
+    if (aux) TP_TRY(obstacle_terms(m, p, false, !total, m->erow.as<double>(), nullptr, st));
+    if (!total || obs) TP_TRY(sum_f64(m->erow.as<double>(), m->nf, sums + (total ? 2 : 0), m, st));
+    if (wm) TP_TRY(willmore_eval(m, sums + 1, nullptr, 0.0, st));
+    return read_energy(m, wm, obs, E_host, st);
 }
 
 int differential_dev(tp_mesh* m, const tp_params* p, double* dE, double* E_host, cudaStream_t st,
                      bool aux) {
     TP_TRY(ensure(m->adj, sizeof(double) * 7 * (size_t)m->nf));
     TP_TRY(ensure(m->erow, sizeof(double) * m->nf));
-    if (p->theta > 0.0)
-        TP_TRY(diff_adjoints_bh(m, p, m->adj.as<double>(), m->erow.as<double>(), st));
-    else
-        TP_TRY(diff_adjoints_direct(m, p, m->adj.as<double>(), m->erow.as<double>(), st));
-    if (aux)
-        TP_TRY(obstacle_terms(m, p, true, true, m->erow.as<double>(), m->adj.as<double>(), st));
-    TP_TRY(adjoints_to_dE(m, m->adj.as<double>(), dE, st));
     TP_TRY(ensure(m->rowsum, sizeof(double) * 8));
-    const bool wm = aux && m->willmore_w > 0.0;
-    if (wm) TP_TRY(willmore_eval(m, m->rowsum.as<double>() + 1, dE, m->willmore_w, st));
+    double* sums = m->rowsum.as<double>();
+    const bool wm = aux && m->willmore_w > 0.0, obs = aux && m->obs;
+    // (an obstacle adds to the face adjoints, so they are kept then)
+    const bool fused = p6_fp32_direct(p) && !obs;
+    if (fused) {
+        TP_TRY(ensure(m->corner, sizeof(double) * 9 * (size_t)m->nf));
+        TP_TRY(diff_p6(m, nullptr, nullptr, m->corner.as<double>(), sums, st));
+        TP_TRY(corners_to_vertices(m, m->corner.as<double>(), 3, dE, st));
+    } else {
+        if (p->theta > 0.0)
+            TP_TRY(diff_adjoints_bh(m, p, m->adj.as<double>(), m->erow.as<double>(), st));
+        else if (p6_fp32_direct(p))
+            TP_TRY(diff_p6(m, m->adj.as<double>(), m->erow.as<double>(), nullptr, nullptr, st));
+        else
+            TP_TRY(diff_adjoints_direct(m, p, m->adj.as<double>(), m->erow.as<double>(), st));
+        if (obs) TP_TRY(obstacle_terms(m, p, true, true, m->erow.as<double>(), m->adj.as<double>(), st));
+        TP_TRY(adjoints_to_dE(m, m->adj.as<double>(), dE, st));
+    }
+    if (wm) TP_TRY(willmore_eval(m, sums + 1, dE, m->willmore_w, st));
     if (E_host) {
-        TP_TRY(sum_f64(m->erow.as<double>(), m->nf, m->rowsum.as<double>(), m, st));
-        double r[2] = {0.0, 0.0};
-        TP_CUDA(cudaMemcpyAsync(r, m->rowsum.ptr, sizeof(double) * (wm ? 2 : 1), cudaMemcpyDeviceToHost, st));
-        TP_CUDA(cudaStreamSynchronize(st));
-        *E_host = r[0] + (wm ? m->willmore_w * r[1] : 0.0);
+        if (!fused) TP_TRY(sum_f64(m->erow.as<double>(), m->nf, sums, m, st));
+        TP_TRY(read_energy(m, wm, false, E_host, st));
     }
     return TP_OK;
 }

@@ -433,6 +433,14 @@ int apply_tc_error(tp_mesh* m, int* gave_up, cudaStream_t st);
 int apply_op(tp_mesh* m, const tp_params* p, int op, const double* v_dev, int k, double* y_dev,
              cudaStream_t st);
 
+// -------- energy.cu --------------------------------------------------------
+// direct sums in FP32 at p = 6 (the default mode): whether p asks for them
+bool p6_fp32_direct(const tp_params* p);
+int energy_total_p6(tp_mesh* m, double* E_dev, cudaStream_t st);   // E of Eq. 10 into a device scalar
+// the face corners' gradients [nf*9] and E (device), or with corner = nullptr the
+// face adjoints [nf*7] and energy rows
+int diff_p6(tp_mesh* m, double* adj, double* erow, double* corner, double* E_dev, cudaStream_t st);
+
 // -------- bvh.cu -----------------------------------------------------------
 int bvh_build(tp_mesh* m, const tp_params* p, cudaStream_t st);
 int energy_rows_bh(tp_mesh* m, const tp_params* p, const int32_t* targets_dev, int nt,
