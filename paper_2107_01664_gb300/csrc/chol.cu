@@ -82,6 +82,7 @@ struct CholState {
     // (small_n nodes, small_lvls levels)
     size_t solve_smem[CH_KMAX + 1] = {}, small_smem[CH_KMAX + 1] = {};
     int small_n[CH_KMAX + 1] = {};
+    bool wide = false;         // a front has more than 256 rows, or CHN_DIRECT
     Buf L, U, uvec, ybuf, xbuf, ctl, part, x, r, bp;
     bool factored = false;
     int ncomp = 1;
@@ -634,7 +635,7 @@ struct StepSmem {
 // depend on the children (factor block to shared memory, w = (r_J ; 0),
 // the children's records); fwd_finish adds the children's update vectors
 // and forms y_J = L11^-1 w_J and u_J = w_S - L21 y_J.
-template <int K>
+template <int K, bool WIDE>
 __device__ __forceinline__ void fwd_prepare(const SweepArgs& A, const CholNode& nd, float* smem, ChildRec* kids) {
     constexpr int KP = Kp<K>::P;
     const int n = nd.nJ, t = nd.t, tid = threadIdx.x;
@@ -646,7 +647,7 @@ __device__ __forceinline__ void fwd_prepare(const SweepArgs& A, const CholNode& 
                       [&](int e) { const int a = e / K; return a < n ? (float)__ldcg(A.r + (size_t)perm[a] * K + (e - a * K)) : 0.f; },
                       [&](int e, float v) { const int a = e / K; w[a * KP + (e - a * K)] = v; });
     const int nc = nd.child1 - nd.child0;
-    if (nc <= CH_MAXCH && !(nd.flags & CHN_DIRECT)) {
+    if (nc <= CH_MAXCH && !(WIDE && (nd.flags & CHN_DIRECT))) {
         // the children's records, then their target rows in this front
         if (tid == 0) {
             int row0 = 0;
@@ -664,7 +665,7 @@ __device__ __forceinline__ void fwd_prepare(const SweepArgs& A, const CholNode& 
     }
 }
 
-template <int K>
+template <int K, bool WIDE>
 __device__ void fwd_finish(const SweepArgs& A, const CholNode& nd, float* smem, const ChildRec* kids) {
     constexpr int KP = Kp<K>::P;
     const int n = nd.nJ, m = nd.mJ, t = nd.t, tid = threadIdx.x;
@@ -675,7 +676,7 @@ __device__ void fwd_finish(const SweepArgs& A, const CholNode& nd, float* smem, 
     const float* Li = smem;       // n x n, leading dimension ldn
     const float* L21 = smem + n * ldn;   // m x n, leading dimension ldm
     const int nc = nd.child1 - nd.child0;
-    if (nc <= CH_MAXCH && !(nd.flags & CHN_DIRECT)) {
+    if (nc <= CH_MAXCH && !(WIDE && (nd.flags & CHN_DIRECT))) {
         // every child's update vector in one batched pass, then the
         // extend-add from shared memory, one child at a time
         const int rows = nc ? kids[nc - 1].row0 + kids[nc - 1].mJ : 0;
@@ -703,12 +704,19 @@ __device__ void fwd_finish(const SweepArgs& A, const CholNode& nd, float* smem, 
             const CholNode cn = A.nodes[A.child_idx[nd.child0 + ci]];
             const int* rl = A.rel + cn.s0;
             const float* uc = A.uvec + (size_t)cn.voff * K;
-            const bool same = nd.flags & CHN_INPLACE;   // the child's rows are this front's
-            gather_batched<12>(cn.mJ * K, [&](int e) { return __ldcg(uc + e); },
-                               [&](int e, float v) {
-                                   const int x = e / K;
-                                   w[(same ? x : __ldg(rl + x)) * KP + (e - x * K)] += v;
-                               });
+            if constexpr (WIDE) {
+                const bool same = nd.flags & CHN_INPLACE;   // the child's rows are this front's
+                gather_batched<12>(cn.mJ * K, [&](int e) { return __ldcg(uc + e); },
+                                   [&](int e, float v) {
+                                       const int x = e / K;
+                                       w[(same ? x : __ldg(rl + x)) * KP + (e - x * K)] += v;
+                                   });
+            } else {
+                for (int idx = tid; idx < cn.mJ * K; idx += CHS_T) {
+                    const int x = idx / K, c = idx - x * K;
+                    w[rl[x] * KP + c] += __ldcg(uc + idx);
+                }
+            }
             __syncthreads();
         }
     }
@@ -726,7 +734,7 @@ __device__ void fwd_finish(const SweepArgs& A, const CholNode& nd, float* smem, 
         for (int c = 0; c < K; ++c) uj[r * K + c] = w[(n + r) * KP + c] - acc[c];
     };
     // (two passes of 128 rows or fewer keep both halves of the block on a row)
-    if (m > 256)
+    if (WIDE && m > 256)
         tall_matvec<K>(L21, ldm, m, n, y, put_u);
     else
         rows_matvec<K>(L21, 1, ldm, m, n, 2, y, sm.scratch, put_u);
@@ -747,7 +755,7 @@ __device__ __forceinline__ void bwd_prepare(const SweepArgs& A, const CholNode& 
     for (int x = threadIdx.x; x < nd.mJ; x += CHS_T) sm.aux[x] = A.struct_pos[nd.s0 + x];
 }
 
-template <int K>
+template <int K, bool WIDE>
 __device__ void bwd_finish(const SweepArgs& A, const CholNode& nd, float* smem) {
     constexpr int KP = Kp<K>::P;
     const int n = nd.nJ, m = nd.mJ, tid = threadIdx.x;
@@ -783,7 +791,7 @@ __device__ void bwd_finish(const SweepArgs& A, const CholNode& nd, float* smem) 
     };
     // rows_matvec takes about 15 cycles per term of its longest thread, m / 2 terms;
     // the lanes' sums about 30 per column and row, n / 8 rows a warp
-    if (m > 4 * n && m > 128)
+    if (WIDE && m > 4 * n && m > 128)
         wide_matvec<K>(L21, ldm, n, m, xs, put_z);
     else
         rows_matvec<K>(L21, ldm, 1, n, m, 2, xs, sm.scratch, put_z);
@@ -841,7 +849,10 @@ __device__ bool wait_until(const unsigned* p, unsigned target, bool at_least, Ch
 // many blocks are resident. Flags hold the sweep's epoch, so they need no
 // reset; the last block to finish the residual resets the counters and
 // advances the epoch.
-template <int K>
+// WIDE: the tree has fronts of more than 256 rows (their matvecs, and vectors of the
+// children read in place). Without those paths the kernel is 1 to 4 us shorter a
+// sweep on meshes of 1,000 to 10,000 vertices.
+template <int K, bool WIDE>
 __global__ void __launch_bounds__(CHS_T)
 k_chol_sweep(SweepArgs A) {
     CholCtl* ctl = A.ctl;
@@ -868,7 +879,7 @@ k_chol_sweep(SweepArgs A) {
         const int J = fwd ? A.order[tk] : A.order[2 * nn - 1 - tk];
         const CholNode nd = A.nodes[J];
         if (fwd)
-            fwd_prepare<K>(A, nd, smem, s_kids);
+            fwd_prepare<K, WIDE>(A, nd, smem, s_kids);
         else
             bwd_prepare<K>(A, nd, smem);
         // wait: forward for every child (one thread each), backward for the
@@ -888,9 +899,9 @@ k_chol_sweep(SweepArgs A) {
         CH_TRACE(tk, 2);
         if (s_ok) {
             if (fwd)
-                fwd_finish<K>(A, nd, smem, s_kids);
+                fwd_finish<K, WIDE>(A, nd, smem, s_kids);
             else
-                bwd_finish<K>(A, nd, smem);
+                bwd_finish<K, WIDE>(A, nd, smem);
         }
         __syncthreads();
         CH_TRACE(tk, 3);
@@ -1192,7 +1203,8 @@ static int upload(Buf& b, const std::vector<T>& v) {
 
 template <int K>
 static int solve_smem_attr() {
-    TP_CUDA(cudaFuncSetAttribute(k_chol_sweep<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CH_SMEM_MAX));
+    TP_CUDA(cudaFuncSetAttribute(k_chol_sweep<K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CH_SMEM_MAX));
+    TP_CUDA(cudaFuncSetAttribute(k_chol_sweep<K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CH_SMEM_MAX));
     if constexpr (K < CH_KMAX) return solve_smem_attr<K + 1>();
     return TP_OK;
 }
@@ -1252,6 +1264,7 @@ static int chol_setup(tp_mesh* m) {
             // a chain's link reads one vector in order, and a front whose children
             // do not fit beside it reads theirs from global memory
             if ((flags[J] & CHN_INPLACE) || step_smem(J, CH_KMAX, false) > CH_SMEM_MAX) flags[J] |= CHN_DIRECT;
+            c->wide = c->wide || (flags[J] & CHN_DIRECT) || mm > 256;
             for (int K = 1; K <= CH_KMAX; ++K)
                 lvl_smem[K] = std::max(lvl_smem[K], step_smem(J, K, flags[J] & CHN_DIRECT));
             // partial Cholesky, Schur update of struct x struct, triangular inverse
@@ -1471,7 +1484,11 @@ static int chol_sweep_kernels(tp_mesh* m, int nsweep, int rgrid, double* partr, 
             const int want = !parts ? nn : part == 1 ? nn - small : small;
             const int grid = std::max(1, std::min(want, most));
             if (want == 0) continue;
-            k_chol_sweep<K><<<grid, CHS_T, big ? c->solve_smem[K] : c->small_smem[K], st>>>(A);
+            const size_t smem = big ? c->solve_smem[K] : c->small_smem[K];
+            if (c->wide)
+                k_chol_sweep<K, true><<<grid, CHS_T, smem, st>>>(A);
+            else
+                k_chol_sweep<K, false><<<grid, CHS_T, smem, st>>>(A);
             TP_CUDA(cudaGetLastError());
             ++*nk;
         }
