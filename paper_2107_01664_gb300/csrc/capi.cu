@@ -277,6 +277,7 @@ int tp_mesh_destroy(tp_mesh* m) {
     release(m->bhl_cnt);
     release(m->bhl_far);
     release(m->bhl_near);
+    release(m->bhl_pool);
     prof_release(m);
     for (auto& b : m->tmpv) release(b);
     for (auto& b : m->stepv) release(b);

@@ -783,40 +783,44 @@ int diff_adjoints_direct(tp_mesh* m, const tp_params* p, double* adj, double* er
 //   X = (f_i+f_j+f_k)/3, n = (f_j-f_i) x (f_k-f_i), a = |n|/2, N = n/|n|;
 //   w = (I - N N^T) gN / |n| + ga N / 2;  g_j = e2 x w, g_k = w x e1,
 //   g_i = -(g_j + g_k), plus gX/3 on each corner.
-__global__ void k_adj_to_corner(const double* __restrict__ pos, const int* __restrict__ faces,
-                                int nf, const double* __restrict__ adj, double* __restrict__ corner) {
-    int S = blockIdx.x * blockDim.x + threadIdx.x;
+// (N and |n| = 2 a from the face tables, one reciprocal for the divisions by |n|: the
+// FP64 pipe bounds this kernel, 83 -> 42 us on 327,680 faces)
+__global__ void __launch_bounds__(128)
+k_adj_to_corner(const double* __restrict__ pos, const int* __restrict__ faces, int nf, const d4* __restrict__ f64a,
+                const d4* __restrict__ f64b, const double* __restrict__ adj, double* __restrict__ corner) {
+    const int S = blockIdx.x * blockDim.x + threadIdx.x;
     if (S >= nf) return;
-    int i = faces[3 * S], j = faces[3 * S + 1], k = faces[3 * S + 2];
+    const size_t i = faces[3 * S], j = faces[3 * S + 1], k = faces[3 * S + 2];
     double e1[3], e2[3];
     for (int c = 0; c < 3; ++c) {
         e1[c] = pos[3 * j + c] - pos[3 * i + c];
         e2[c] = pos[3 * k + c] - pos[3 * i + c];
     }
-    double n[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2],
-                   e1[0] * e2[1] - e1[1] * e2[0]};
-    double nn = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-    double N[3] = {n[0] / nn, n[1] / nn, n[2] / nn};
-    const double* g = adj + 7 * S;
-    double gNn = g[3] * N[0] + g[4] * N[1] + g[5] * N[2];
+    const d4 Nq = f64b[S];
+    const double N[3] = {Nq.x, Nq.y, Nq.z}, nn = 2.0 * f64a[S].w;
+    const double rn = nn > 1e-280 && nn < 1e280 ? rcp64(nn) : 1.0 / nn;
+    const double* g = adj + 7 * (size_t)S;
+    const double gNn = g[3] * N[0] + g[4] * N[1] + g[5] * N[2];
     double w[3];
-    for (int c = 0; c < 3; ++c) w[c] = (g[3 + c] - gNn * N[c]) / nn + 0.5 * g[6] * N[c];
-    double gj[3] = {e2[1] * w[2] - e2[2] * w[1], e2[2] * w[0] - e2[0] * w[2],
-                    e2[0] * w[1] - e2[1] * w[0]};
-    double gk[3] = {w[1] * e1[2] - w[2] * e1[1], w[2] * e1[0] - w[0] * e1[2],
-                    w[0] * e1[1] - w[1] * e1[0]};
+    for (int c = 0; c < 3; ++c) w[c] = div64(g[3 + c] - gNn * N[c], nn, rn) + 0.5 * g[6] * N[c];
+    const double gj[3] = {e2[1] * w[2] - e2[2] * w[1], e2[2] * w[0] - e2[0] * w[2],
+                          e2[0] * w[1] - e2[1] * w[0]};
+    const double gk[3] = {w[1] * e1[2] - w[2] * e1[1], w[2] * e1[0] - w[0] * e1[2],
+                          w[0] * e1[1] - w[1] * e1[0]};
+    double* cr = corner + 9 * (size_t)S;
     for (int c = 0; c < 3; ++c) {
-        double third = g[c] / 3.0;
-        corner[9 * S + c] = -(gj[c] + gk[c]) + third;
-        corner[9 * S + 3 + c] = gj[c] + third;
-        corner[9 * S + 6 + c] = gk[c] + third;
+        const double third = third64(g[c]);
+        cr[c] = -(gj[c] + gk[c]) + third;
+        cr[3 + c] = gj[c] + third;
+        cr[6 + c] = gk[c] + third;
     }
 }
 
 int adjoints_to_dE(tp_mesh* m, const double* adj, double* dE, cudaStream_t st) {
     TP_TRY(ensure(m->corner, sizeof(double) * 9 * (size_t)m->nf));
-    k_adj_to_corner<<<(m->nf + 255) / 256, 256, 0, st>>>(m->pos.as<double>(), m->faces.as<int>(),
-                                                         m->nf, adj, m->corner.as<double>());
+    k_adj_to_corner<<<(m->nf + 127) / 128, 128, 0, st>>>(m->pos.as<double>(), m->faces.as<int>(), m->nf,
+                                                         m->f64a.as<d4>(), m->f64b.as<d4>(), adj,
+                                                         m->corner.as<double>());
     TP_LAUNCH_CHECK();
     return corners_to_vertices(m, m->corner.as<double>(), 3, dE, st);
 }
@@ -2267,52 +2271,59 @@ __device__ __forceinline__ float4 f4add(float4 a, float4 b) {
 }
 
 // node sums of X and (PROJ) node-average projectors (upper triangle xx, xy,
-// xz, yy, yz, zz in two float4), one depth level per launch, deepest first
+// xz, yy, yz, zz in two float4), from the leaves up in one launch: a thread per
+// (leaf, float4 of X or the projector), of the two that arrive at an inner node for
+// one part the second (flags, zero before) goes on, and a part of a node is the sum of
+// its children's in a fixed order. 327,680 faces, 3 columns: one launch per tree level
+// took 107 us, now 52 us.
 template <int NW4, bool PROJ>
-__global__ void k_node_X(const BvhNode* __restrict__ node, const int* __restrict__ right,
-                         const int* __restrict__ order, int n0, int n1, const float4* __restrict__ Ws,
-                         const float4* __restrict__ sa, const float4* __restrict__ sb,
-                         float4* __restrict__ nodeX, float4* __restrict__ nodeP) {
-    const int k = n0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n1) return;
-    const int id = order[k];
-    const BvhNode n = node[id];
-    float4 acc[NW4];
-#pragma unroll
-    for (int q = 0; q < NW4; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    float P[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (n.leaf) {
-        float asum = 0.f;
-        for (int i = n.first; i < n.first + n.count; ++i) {
-#pragma unroll
-            for (int q = 0; q < NW4; ++q) acc[q] = f4add(acc[q], Ws[(size_t)i * NW4 + q]);
-            if (PROJ) {
-                const float a = sa[i].w;
-                const float4 N = sb[i];
-                P[0] += a * N.x * N.x; P[1] += a * N.x * N.y; P[2] += a * N.x * N.z;
-                P[3] += a * N.y * N.y; P[4] += a * N.y * N.z; P[5] += a * N.z * N.z;
-                asum += a;
+__global__ void __launch_bounds__(128)
+k_node_X(const BvhNode* __restrict__ node, int nleaf, const float4* __restrict__ Ws, const float4* __restrict__ sa,
+         const float4* __restrict__ sb, float4* nodeX, float4* nodeP, unsigned* __restrict__ flags) {
+    constexpr int Q = NW4 + (PROJ ? 1 : 0);
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, lf = t / Q, q = t - lf * Q;
+    if (lf >= nleaf) return;
+    int path[BVH_MAXDEPTH], depth = 0;
+    walk_to_leaf(lf, nleaf, [&](int id) { path[depth++] = id; });
+    const bool proj = PROJ && q == NW4;
+    for (int d = depth - 1; d >= 0; --d) {
+        const int id = path[d];
+        if (d == depth - 1) {
+            const int first = node[id].first, count = node[id].count;
+            if (!proj) {
+                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int i = first; i < first + count; ++i) acc = f4add(acc, Ws[(size_t)i * NW4 + q]);
+                nodeX[(size_t)id * NW4 + q] = acc;
+            } else {
+                float P[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, asum = 0.f;
+                for (int i = first; i < first + count; ++i) {
+                    const float a = sa[i].w;
+                    const float4 N = sb[i];
+                    P[0] += a * N.x * N.x; P[1] += a * N.x * N.y; P[2] += a * N.x * N.z;
+                    P[3] += a * N.y * N.y; P[4] += a * N.y * N.z; P[5] += a * N.z * N.z;
+                    asum += a;
+                }
+                for (int c = 0; c < 6; ++c) P[c] /= asum;
+                nodeP[2 * (size_t)id] = make_float4(P[0], P[1], P[2], P[3]);
+                nodeP[2 * (size_t)id + 1] = make_float4(P[4], P[5], 0.f, 0.f);
             }
+            continue;
         }
-        if (PROJ)
-            for (int c = 0; c < 6; ++c) P[c] /= asum;
-    } else {
-        const int L = id + 1, R = right[id];
-#pragma unroll
-        for (int q = 0; q < NW4; ++q) acc[q] = f4add(nodeX[(size_t)L * NW4 + q], nodeX[(size_t)R * NW4 + q]);
-        if (PROJ) {
+        __threadfence();
+        if (atomicAdd(flags + (size_t)id * Q + q, 1u) == 0u) return;
+        __threadfence();
+        const int L = id + 1, R = bvh_right(id, node[id].skip);
+        if (!proj) {
+            nodeX[(size_t)id * NW4 + q] =
+                f4add(__ldcg(nodeX + (size_t)L * NW4 + q), __ldcg(nodeX + (size_t)R * NW4 + q));
+        } else {
             const float aL = node[L].a, aR = node[R].a, ia = 1.f / (aL + aR);
-            const float4 l0 = nodeP[2 * L], l1 = nodeP[2 * L + 1], r0 = nodeP[2 * R], r1 = nodeP[2 * R + 1];
-            P[0] = (aL * l0.x + aR * r0.x) * ia; P[1] = (aL * l0.y + aR * r0.y) * ia;
-            P[2] = (aL * l0.z + aR * r0.z) * ia; P[3] = (aL * l0.w + aR * r0.w) * ia;
-            P[4] = (aL * l1.x + aR * r1.x) * ia; P[5] = (aL * l1.y + aR * r1.y) * ia;
+            const float4 l0 = __ldcg(nodeP + 2 * (size_t)L), l1 = __ldcg(nodeP + 2 * (size_t)L + 1),
+                         r0 = __ldcg(nodeP + 2 * (size_t)R), r1 = __ldcg(nodeP + 2 * (size_t)R + 1);
+            nodeP[2 * (size_t)id] = make_float4((aL * l0.x + aR * r0.x) * ia, (aL * l0.y + aR * r0.y) * ia,
+                                                (aL * l0.z + aR * r0.z) * ia, (aL * l0.w + aR * r0.w) * ia);
+            nodeP[2 * (size_t)id + 1] = make_float4((aL * l1.x + aR * r1.x) * ia, (aL * l1.y + aR * r1.y) * ia, 0.f, 0.f);
         }
-    }
-#pragma unroll
-    for (int q = 0; q < NW4; ++q) nodeX[(size_t)id * NW4 + q] = acc[q];
-    if (PROJ) {
-        nodeP[2 * id] = make_float4(P[0], P[1], P[2], P[3]);
-        nodeP[2 * id + 1] = make_float4(P[4], P[5], 0.f, 0.f);
     }
 }
 
@@ -2467,6 +2478,9 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// Four warps (groups) a block: neighbouring groups name the same nodes, whose records
+// then come from L1 (one-warp blocks: 3 columns of A on 327,680 faces 1,805 -> 1,837 us,
+// 9 of B 2,453 -> 2,869).
 template <int OP, int KC>
 __global__ void __launch_bounds__(128)
 k_bh_apply_list(const float4* __restrict__ node4, const float4* __restrict__ nodelo, const float4* __restrict__ sa,
@@ -2653,10 +2667,12 @@ static int launch_bh_apply_op(tp_mesh* m, const tp_params* p, const double* v, i
     TP_TRY(ensure(m->wv64, sizeof(double) * 4 * KC * (size_t)nf));
     TP_TRY(ensure(m->wv32, sizeof(float4) * NW4 * (size_t)nf));
     TP_TRY(ensure(m->corner, sizeof(double) * 3 * (size_t)nf * k));
-    TP_TRY(ensure(m->bh_apply_ws, sizeof(float4) * ((size_t)NW4 * nf + (size_t)NW4 * nn + 2 * (size_t)nn)));
+    TP_TRY(ensure(m->bh_apply_ws, sizeof(float4) * ((size_t)NW4 * nf + (size_t)NW4 * nn + 2 * (size_t)nn) +
+                                      sizeof(unsigned) * (size_t)(NW4 + 1) * nn));
     float4* Ws = m->bh_apply_ws.as<float4>();
     float4* nodeX = Ws + (size_t)NW4 * nf;
     float4* nodeP = nodeX + (size_t)NW4 * nn;
+    unsigned* flags = reinterpret_cast<unsigned*>(nodeP + 2 * (size_t)nn);   // arrivals of k_node_X
     TP_TRY(bh_counter(m, st));
     unsigned long long* cnt = m->bhcount.as<unsigned long long>() + 2;
     BhLists Ls;
@@ -2669,12 +2685,12 @@ static int launch_bh_apply_op(tp_mesh* m, const tp_params* p, const double* v, i
         TP_LAUNCH_CHECK();
         k_sort_X<NW4><<<(nf + 255) / 256, 256, 0, st>>>(m->wv32.as<float4>(), bv.perm, nf, Ws);
         TP_LAUNCH_CHECK();
-        for (int d = bv.maxdepth; d >= 0; --d) {
-            const int n0 = bv.level_off[d], n1 = bv.level_off[d + 1];
-            k_node_X<NW4, LOW><<<(n1 - n0 + 127) / 128, 128, 0, st>>>(bv.node, bv.right, bv.level_order, n0, n1,
-                                                                     Ws, bv.sa, bv.sb, nodeX, nodeP);
-            TP_LAUNCH_CHECK();
-        }
+        constexpr int NQ = NW4 + (LOW ? 1 : 0);
+        const int nleaf = (nn + 1) / 2;
+        TP_CUDA(cudaMemsetAsync(flags, 0, sizeof(unsigned) * (size_t)NQ * nn, st));
+        k_node_X<NW4, LOW><<<(unsigned)(((size_t)nleaf * NQ + 127) / 128), 128, 0, st>>>(
+            bv.node, nleaf, Ws, bv.sa, bv.sb, nodeX, nodeP, flags);
+        TP_LAUNCH_CHECK();
         {
             ProfScope ps(m, PK_BH_APPLY, 0.0, st);
             m->prof.cols[PK_BH_APPLY] += KC;

@@ -190,6 +190,33 @@ struct FaceBox {
     float hix, hiy, hiz, a;
 };
 
+// right child of an inner node: its n leaves make 2 n - 1 nodes in pre-order (skip is
+// the first after them), ceil(n / 2) of them on the left
+__device__ __forceinline__ int bvh_right(int id, int skip) { return id + 2 * (((skip - id + 1) / 2 + 1) / 2); }
+
+// Path from the root to leaf lf of a tree over nleaf leaves, by the shape alone: a
+// node over n leaves has its left child (ceil(n / 2) leaves) next to it and its right
+// child 2 ceil(n / 2) further on
+template <class Visit>
+__device__ __forceinline__ void walk_to_leaf(int lf, int nleaf, Visit visit) {
+    int id = 0, lo = 0, n = nleaf;
+    for (;;) {
+        visit(id);
+        if (n == 1) break;
+        const int nl = (n + 1) / 2;
+        if (lf < lo + nl) {
+            id += 1;
+            n = nl;
+        } else {
+            id += 2 * nl;
+            lo += nl;
+            n -= nl;
+        }
+    }
+}
+
+constexpr int BVH_MAXDEPTH = 32;   // 2^30 faces make at most 31 levels
+
 // squared distance between a face box and a node box; max(0, ...) per axis,
 // fixed operation order (the admissibility test of §4.1 is decided in FP32
 // identically by every kernel)
@@ -354,7 +381,7 @@ struct tp_mesh {
     long long bhl_nfar = 0, bhl_nnear = 0;
     unsigned long long bhl_inter = 0;     // interactions of one evaluation over the lists
     bool bhl_failed = false;              // the lists could not be built for this tree (walk kernels serve)
-    tp::Buf bhl_cnt, bhl_far, bhl_near;
+    tp::Buf bhl_cnt, bhl_far, bhl_near, bhl_pool;
     // workspaces
     tp::Buf part, part2, scal, corner, wv64, wv32, tmpv[8];
     tp::Buf io_in, io_out, adj, erow, tlist, rowsum;

@@ -1,0 +1,45 @@
+"""The Barnes-Hut tree and lists where their construction can go wrong: one leaf, one
+full and one partial leaf, leaves of one face, fewer faces than a group of 32 and one
+face more, short and long lists in turn, and rebuilds on the same mesh. The tree decides in FP32 as the oracle's does, so E, dE and the applies agree
+with the oracle's Barnes-Hut sums over the same tree to the FP32 tolerance, 1e-5."""
+import numpy as np
+import pytest
+
+from oracle import tp_oracle as O
+from synth import small_mesh, vertex_vectors
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-5
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a) - b) / np.linalg.norm(b))
+
+
+@pytest.mark.parametrize("kind", ["tetra", "octa", "torus3x3", "torus8x4", "torus11x3", "torus13x10", "ico3"])
+@pytest.mark.parametrize("leaf", [1, 8, 32])
+@pytest.mark.parametrize("theta", [0.05, 0.5])
+def test_sums_over_the_tree(lib, kind, leaf, theta):
+    V, F = small_mesh(kind, seed=5)
+    u = vertex_vectors(len(V), 3, 8)
+    p = lib.params(theta=theta, leaf_size=leaf)
+    with lib.Mesh(V, F) as m:
+        for _ in range(2):                     # the second time on a tree rebuilt in place
+            E = lib.tp_energy(m, p)
+            g, _ = lib.tp_differential(m, p)
+            y = lib.fractional_apply(m, "A", u, p)
+            m.set_positions(V)
+    assert abs(E / O.bh_energy(V, F, theta, leaf) - 1) <= TOL
+    assert rel(g, O.bh_differential(V, F, theta, leaf)) <= TOL
+    assert rel(y, O.bh_apply_operator(V, F, u, "A", theta, leaf)) <= TOL
+
+
+def test_lists_of_different_length_on_one_mesh(lib):
+    # the pool of one mesh serves short and long lists in turn; at theta = 0.02 nearly
+    # every pair is summed exactly
+    V, F = small_mesh("torus61x33", seed=9)
+    with lib.Mesh(V, F) as m:
+        e = [lib.tp_energy(m, lib.params(theta=t, leaf_size=1)) for t in (1.0, 0.02, 0.5, 0.02)]
+    E = O.energy(V, F)
+    assert e[1] == e[3]
+    assert abs(e[1] / E - 1) <= TOL
