@@ -48,7 +48,7 @@ def flops_per_pair(name, stat):
         kc = stat.get("columns", 0.0) / max(1, stat["launches"]) or 3.0
         return APPLY_FLOPS[name](kc)
     return None
-KERNEL_SOURCE = {"energy_direct": "pairs.cu", "diff_direct": "pairs.cu", "apply_A": "pairs.cu",
+KERNEL_SOURCE = {"energy_direct": "energy.cu", "diff_direct": "energy.cu", "apply_A": "pairs.cu",
                  "apply_B": "pairs.cu", "apply_B0": "pairs.cu", "apply_L": "pairs.cu",
                  "bh_energy": "bvh.cu", "bh_diff": "bvh.cu", "bh_apply": "pairs.cu", "cg": "cg.cu",
                  "bvh_build": "bvh.cu",
