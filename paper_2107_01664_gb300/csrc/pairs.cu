@@ -1095,8 +1095,8 @@ k_apply(const d4* __restrict__ fa, const d4* __restrict__ fb, const d4* __restri
 // tiles of the block's own targets made the runs that meet two of them late (643 us
 // against 608). Per apply at 19,920 faces, k = 3 / 6 / 9, before (three columns in scalar
 // arithmetic, six padded to nine, splits of the sources in several waves) and now:
-//   A  669 / 971 / 970 -> 581 / 774 / 902 us    B  390 / 659 / 659 -> 354 / 512 / 637
-//   B0 451 / 502 / 502 -> 386 / 447 / 479       L  275 / 349 / 349 -> 248 / 300 / 342
+//   A  669 / 971 / 970 -> 579 / 774 / 902 us    B  390 / 659 / 659 -> 355 / 510 / 637
+//   B0 451 / 502 / 502 -> 388 / 449 / 477       L  275 / 349 / 349 -> 250 / 300 / 340
 
 constexpr int WT = 2;   // targets per thread of the wide kernel
 
@@ -1455,25 +1455,15 @@ k_wide_combine(const float2* __restrict__ part, int nf, long long ntiles, long l
 #pragma unroll
         for (int q = 0; q < 3; ++q) at[q] = area ? 0 : 1 + q * KC + c;
         at[3] = L::NH + (area ? 0 : 1 + c);
-        // four slots' loads in flight: a small mesh has as many slots as tiles, and one memory
-        // latency for each made its applies late (A, 1 / 9 columns, 2,400 faces, one call with
-        // its synchronisation: 80 / 91 -> 67 / 78 us; 19,920 faces, 9 columns: 909 -> 902)
-        for (int s0 = 0; s0 < slots; s0 += 4) {
-            float2 x[4][4];
+#pragma unroll 4
+        for (int s = 0; s < slots; ++s) {
+            const float2* ps = part + (size_t)s * L::NA * nf + S;
+            if (L::HIGH) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float2* ps = part + (size_t)(s0 + i) * L::NA * nf + S;
-                const bool in = s0 + i < slots;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const bool use = q < 3 ? L::HIGH && (q == 0 || !area) : L::USEU;
-                    x[i][q] = in && use ? ps[(size_t)at[q] * nf] : make_float2(0.f, 0.f);
-                }
+                for (int q = 0; q < 3; ++q)
+                    if (q == 0 || !area) v[q].add(ps[(size_t)at[q] * nf]);
             }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) v[q].add(x[i][q]);
+            if (L::USEU) v[3].add(ps[(size_t)at[3] * nf]);
         }
     }
     if (area) {
