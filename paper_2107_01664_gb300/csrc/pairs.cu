@@ -837,14 +837,13 @@ int adjoints_to_dE(tp_mesh* m, const double* adj, double* dE, cudaStream_t st) {
 // Per source face the pair kernels read one vector X of NA values: [a, W_V]
 // (the operators with the high-order part) then [a, W_U] (those with a
 // low-order part); accumulator i gains h X[i], with h the high-order kernel
-// on the first NH entries and the low-order one on the rest. Parts of an odd number
-// of entries (KC = 6) end with a zero: NH and NA are
+// on the first NH entries and the low-order one on the rest. NH and NA are
 // even, so the pairs of packed FP32 arithmetic never straddle the parts.
 template <int OP, int KC> struct OpLayout {
     static constexpr bool HIGH = (OP == TP_OP_A || OP == TP_OP_B);
     static constexpr bool USEU = (OP != TP_OP_B);
-    static constexpr int NH = HIGH ? (1 + 3 * KC + 1) / 2 * 2 : 0;   // high-order entries [a, W_V]
-    static constexpr int NL = USEU ? (1 + KC + 1) / 2 * 2 : 0;       // low-order entries [a, W_U]
+    static constexpr int NH = HIGH ? 1 + 3 * KC : 0;          // high-order entries [a, W_V]
+    static constexpr int NL = USEU ? 1 + KC : 0;              // low-order entries [a, W_U]
     static constexpr int NA = NH + NL;                        // accumulators = X entries
     static constexpr int NW4 = (NA + 3) / 4;                  // X in 4-vectors
     static_assert(NH % 2 == 0 && NA % 2 == 0, "pairs of accumulators stay within a part");
@@ -876,7 +875,7 @@ __global__ void k_face_W(const double* __restrict__ v, int k, int col0, const in
     double* w64 = W64 + 4 * KC * (size_t)S;
     T* out = reinterpret_cast<T*>(Wp) + (size_t)S * 4 * nw4;
     const bool hi = (op == TP_OP_A || op == TP_OP_B), lo = op != TP_OP_B;
-    const int ou = hi ? (1 + 3 * KC + 1) / 2 * 2 : 0;   // start of the low-order block in out
+    const int ou = hi ? 1 + 3 * KC : 0;   // start of the low-order block in out
     // the FP64 kernel leaves the factor 1/2 of the low-order kernel to X (exact)
     const double half = sizeof(T) == 8 && (op == TP_OP_A || op == TP_OP_B0) ? 0.5 : 1.0;
     for (int c = 0; c < CG && c0 + c < KC; ++c) {
@@ -893,7 +892,6 @@ __global__ void k_face_W(const double* __restrict__ v, int k, int col0, const in
     }
     if (g == 0) {
         if (hi) out[0] = (T)a;
-        if (hi && KC % 2 == 0) out[ou - 1] = T(0);
         if (lo) out[ou] = (T)(half * a);
         for (int n = ou + (lo ? 1 + KC : 0); n < 4 * nw4; ++n) out[n] = T(0);
     }
@@ -972,8 +970,7 @@ __device__ __forceinline__ typename P2T<T>::type p2zero() {
 // One (target, source) term of the kernel-matrix products on the source's
 // vector X (pairs x2[i] = X[2i], X[2i+1]). SELF = the tile may contain the
 // target itself (d = 0), whose term must be dropped: the kernels of B and
-// L^{2-s} do not vanish at d = 0 by themselves (FP64 only: k_apply_wide tests in
-// its own chunks).
+// L^{2-s} do not vanish at d = 0 by themselves.
 template <typename T, int OP, bool SELF, int KC>
 __device__ __forceinline__ void apply_term(T dx, T dy, T dz, T nx, T ny, T nz, T mx, T my, T mz,
                                            const typename P2T<T>::type* x2, T s_exp, T l_exp,
@@ -998,11 +995,13 @@ __device__ __forceinline__ void apply_term(T dx, T dy, T dz, T nx, T ny, T nz, T
         return;
     }
     if (OP == TP_OP_L) {
-        const T h = pow_(r2, -l_exp);
+        T h = pow_(r2, -l_exp);
+        if (SELF) h = r2 > T(2) * tiny_r2<T>() ? h : T(0);
 #pragma unroll
         for (int i = 0; i < L::NA / 2; ++i) pt[i] = pfma(h, x2[i], pt[i]);
     } else {
-        const T hB = pow_(r2, -s_exp);
+        T hB = pow_(r2, -s_exp);
+        if (SELF) hB = r2 > T(2) * tiny_r2<T>() ? hB : T(0);
 #pragma unroll
         for (int i = 0; i < L::NH / 2; ++i) pt[i] = pfma(hB, x2[i], pt[i]);
         if (LOW) {
@@ -1016,87 +1015,149 @@ __device__ __forceinline__ void apply_term(T dx, T dy, T dz, T nx, T ny, T nz, T
     }
 }
 
-// the FP64 path, one target a thread (the FP32 path is k_apply_wide)
-template <int OP, int KC>
+template <typename T, int OP, int TT, int KC>
 __global__ void __launch_bounds__(NT)
-k_apply(const d4* __restrict__ fa, const d4* __restrict__ fb, const d4* __restrict__ Wp, int nf, int tiles_per_split,
-        double* __restrict__ part, RootPow rp) {
+k_apply(const typename V4T<T>::type* __restrict__ fa, const typename V4T<T>::type* __restrict__ fb,
+        const float4* __restrict__ flo, const float4* __restrict__ tbox, const double* __restrict__ center,
+        const typename V4T<T>::type* __restrict__ Wp, int nf, int tiles_per_split, T s_exp,
+        T l_exp, double* __restrict__ part, RootPow rp) {
+    using V4 = typename V4T<T>::type;
     using L = OpLayout<OP, KC>;
     constexpr bool LOW = (OP == TP_OP_A || OP == TP_OP_B0);
-    __shared__ d4 sa[NT];
-    __shared__ d4 sb[LOW ? NT : 1];
-    __shared__ d4 sw[NT * L::NW4];
-    const int t = blockIdx.x * NT + threadIdx.x;
-    const bool has = t < nf;
-    const d4 A = has ? fa[t] : v4zero<double>(), B = LOW && has ? fb[t] : v4zero<double>();
+    constexpr bool F32 = sizeof(T) == 4;
+    __shared__ V4 sa[NT];
+    __shared__ V4 sb[LOW ? NT : 1];
+    __shared__ V4 sw[NT * L::NW4];
+    __shared__ float4 shl[F32 ? NT : 1];
+    __shared__ float sbox[6];
+    T tx[TT], ty[TT], tz[TT], nx[TT], ny[TT], nz[TT];
+    float lx[TT], ly[TT], lz[TT];
+    int tid[TT];
+    float bl[3] = {3e38f, 3e38f, 3e38f}, bh[3] = {-3e38f, -3e38f, -3e38f};
+#pragma unroll
+    for (int j = 0; j < TT; ++j) {
+        const int t = blockIdx.x * NT * TT + j * NT + threadIdx.x;
+        tid[j] = t;
+        tx[j] = ty[j] = tz[j] = nx[j] = ny[j] = nz[j] = T(0);
+        lx[j] = ly[j] = lz[j] = 0.f;
+        if (t < nf) {
+            V4 A = fa[t];
+            tx[j] = A.x; ty[j] = A.y; tz[j] = A.z;
+            if (LOW) {
+                V4 B = fb[t];
+                nx[j] = B.x; ny[j] = B.y; nz[j] = B.z;
+            }
+            if (F32) {
+                float4 Lo = flo[t];
+                lx[j] = Lo.x; ly[j] = Lo.y; lz[j] = Lo.z;
+                bl[0] = fminf(bl[0], (float)A.x); bl[1] = fminf(bl[1], (float)A.y); bl[2] = fminf(bl[2], (float)A.z);
+                bh[0] = fmaxf(bh[0], (float)A.x); bh[1] = fmaxf(bh[1], (float)A.y); bh[2] = fmaxf(bh[2], (float)A.z);
+            }
+        }
+    }
+    float thr2 = 0.f;
+    if (F32) {
+        block_box(bl[0], bl[1], bl[2], bh[0], bh[1], bh[2], sbox);
+        thr2 = (float)center[3];
+    }
+    using P2 = typename P2T<T>::type;
     constexpr int NP = L::NA / 2;   // accumulator pairs
-    Acc2<double> acc[NP];
+    Acc2<T> acc[TT][NP];
     const int ntiles = (nf + NT - 1) / NT;
     const int k0 = blockIdx.y * tiles_per_split;
     const int k1 = min(k0 + tiles_per_split, ntiles);
     for (int tile = k0; tile < k1; ++tile) {
-        const int src = tile * NT + threadIdx.x;
+        // tiles holding this block's own targets (self pairs) or lying near them
+        // take the careful path: compensated differences and the self-pair test
+        const bool diag = tile >= (int)blockIdx.x * TT && tile < ((int)blockIdx.x + 1) * TT;
+        const bool near = F32 && tile_near(tbox, tile, sbox, thr2);
+        int src = tile * NT + threadIdx.x;
         __syncthreads();
-        sa[threadIdx.x] = src < nf ? fa[src] : v4zero<double>();
-        if (LOW) sb[threadIdx.x] = src < nf ? fb[src] : v4zero<double>();
+        sa[threadIdx.x] = src < nf ? fa[src] : v4zero<T>();
+        if (LOW) sb[threadIdx.x] = src < nf ? fb[src] : v4zero<T>();
+        if (near) shl[threadIdx.x] = src < nf ? flo[src] : make_float4(0.f, 0.f, 0.f, 0.f);
         for (int i = threadIdx.x; i < NT * L::NW4; i += NT) {
-            const int f = tile * NT + i / L::NW4;
-            sw[i] = f < nf ? Wp[(size_t)tile * NT * L::NW4 + i] : v4zero<double>();
+            int f = tile * NT + i / L::NW4;
+            sw[i] = f < nf ? Wp[(size_t)tile * NT * L::NW4 + i] : v4zero<T>();
         }
         __syncthreads();
-        auto chunk = [&](int c, auto own) {   // own: the tile of the block's targets (self-pair test)
-            double2 pt[NP];
+        for (int c = 0; c < NT; c += CH) {
+            P2 pt[TT][NP];
 #pragma unroll
-            for (int i = 0; i < NP; ++i) pt[i] = p2zero<double>();
-#pragma unroll(decltype(own)::value ? 1 : 2)
-            for (int jj = c; jj < c + CH; ++jj) {
-                const d4 s = sa[jj];
-                double2 wv[2 * L::NW4];
+            for (int j = 0; j < TT; ++j)
 #pragma unroll
-                for (int i = 0; i < L::NW4; ++i) {
-                    const d4 x = sw[jj * L::NW4 + i];
-                    wv[2 * i] = make_double2(x.x, x.y);
-                    wv[2 * i + 1] = make_double2(x.z, x.w);
+                for (int i = 0; i < NP; ++i) pt[j][i] = p2zero<T>();
+            if (near || diag) {
+                for (int q = 0; q < CH; ++q) {
+                    const int jj = c + q;
+                    V4 s = sa[jj];
+                    float4 l = near ? shl[jj] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    P2 wv[2 * L::NW4];
+#pragma unroll
+                    for (int i = 0; i < L::NW4; ++i) {
+                        V4 x = sw[jj * L::NW4 + i];
+                        wv[2 * i].x = x.x; wv[2 * i].y = x.y; wv[2 * i + 1].x = x.z; wv[2 * i + 1].y = x.w;
+                    }
+                    T mx = 0, my = 0, mz = 0;
+                    if (LOW) {
+                        V4 n = sb[jj];
+                        mx = n.x; my = n.y; mz = n.z;
+                    }
+#pragma unroll
+                    for (int j = 0; j < TT; ++j)
+                        apply_term<T, OP, true, KC>((tx[j] - s.x) + (T)(lx[j] - l.x), (ty[j] - s.y) + (T)(ly[j] - l.y),
+                                                    (tz[j] - s.z) + (T)(lz[j] - l.z), nx[j], ny[j], nz[j], mx,
+                                                    my, mz, wv, s_exp, l_exp, pt[j], rp);
                 }
-                const d4 n = LOW ? sb[jj] : v4zero<double>();
-                apply_term<double, OP, decltype(own)::value, KC>(A.x - s.x, A.y - s.y, A.z - s.z, B.x, B.y, B.z, n.x,
-                                                                 n.y, n.z, wv, 0.0, 0.0, pt, rp);
+            } else {
+#pragma unroll 2
+                for (int q = 0; q < CH; ++q) {
+                    const int jj = c + q;
+                    V4 s = sa[jj];
+                    P2 wv[2 * L::NW4];
+#pragma unroll
+                    for (int i = 0; i < L::NW4; ++i) {
+                        V4 x = sw[jj * L::NW4 + i];
+                        wv[2 * i].x = x.x; wv[2 * i].y = x.y; wv[2 * i + 1].x = x.z; wv[2 * i + 1].y = x.w;
+                    }
+                    T mx = 0, my = 0, mz = 0;
+                    if (LOW) {
+                        V4 n = sb[jj];
+                        mx = n.x; my = n.y; mz = n.z;
+                    }
+#pragma unroll
+                    for (int j = 0; j < TT; ++j)
+                        apply_term<T, OP, false, KC>(tx[j] - s.x, ty[j] - s.y, tz[j] - s.z, nx[j], ny[j], nz[j],
+                                                     mx, my, mz, wv, s_exp, l_exp, pt[j], rp);
+                }
             }
 #pragma unroll
-            for (int i = 0; i < NP; ++i) acc[i].add(pt[i]);
-        };
-        for (int c = 0; c < NT; c += CH)
-            if (tile == (int)blockIdx.x) chunk(c, std::true_type());
-            else chunk(c, std::false_type());
-    }
-    if (has)
+            for (int j = 0; j < TT; ++j)
 #pragma unroll
-        for (int i = 0; i < L::NA; ++i)
-            part[((size_t)blockIdx.y * L::NA + i) * nf + t] = acc[i / 2].value(i & 1);
+                for (int i = 0; i < NP; ++i) acc[j][i].add(pt[j][i]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < TT; ++j)
+        if (tid[j] < nf)
+#pragma unroll
+            for (int i = 0; i < L::NA; ++i)
+                part[((size_t)blockIdx.y * L::NA + i) * nf + tid[j]] = acc[j][i / 2].value(i & 1);
 }
 
-// ---- FP32 products with two targets per thread -----------------------------
-// Passes of three, six or nine columns (the lockstep solver applies A and L^{2-s}
-// to three right-hand sides of three columns, fewer as they converge). The kernel
-// value of a (target, source) pair is evaluated for both targets
+// ---- 9-column products with two targets per thread -------------------------
+// The FP32 path of the 9-column products (the lockstep solver applies A and
+// L^{2-s} to three right-hand sides at once) takes two targets per thread.
+// The kernel value of a (target, source) pair is evaluated for both targets
 // in packed f32x2 arithmetic, from source geometry staged pre-broadcast in
 // shared memory ({x,x}, {y,y}, ...), and each source vector X is read from
 // shared memory once for both targets. The per-chunk FP32 sums stay in
 // registers; the Kahan pairs that carry them across chunks live in shared
 // memory (one float4 {s.x, s.y, c.x, c.y} per thread, target and accumulator
 // pair), which keeps the registers for the two targets' chunk sums. Tiles
-// near a warp's targets or holding the block's take compensated differences; the
-// latter also test for the self pair.
-//
-// Bound by the FP32 pipe (FP32 operations a pair: 20 + 2 NA for A, 9 + 2 NA for L;
-// MUFU next for L), at about 70 % of its issue slots. Loops of 8 sources in place of
-// 2 hide the MUFU latency at 8 to 20 warps an SM: 608 -> 579 us for A with three columns
-// at 19,920 faces, 926 -> 902 with nine, 274 -> 250 for L with three. A scalar loop for the
-// tiles of the block's own targets made the runs that meet two of them late (643 us
-// against 608). Per apply at 19,920 faces, k = 3 / 6 / 9, before (three columns in scalar
-// arithmetic, six padded to nine, splits of the sources in several waves) and now:
-//   A  669 / 971 / 970 -> 579 / 774 / 902 us    B  390 / 659 / 659 -> 355 / 510 / 637
-//   B0 451 / 502 / 502 -> 388 / 449 / 477       L  275 / 349 / 349 -> 250 / 300 / 340
+// near the block's targets or holding them take the careful scalar path of
+// k_apply (compensated differences, self-pair test). Partial sums leave as
+// FP32 Kahan pairs (s, c), one per split.
 
 constexpr int WT = 2;   // targets per thread of the wide kernel
 
@@ -1107,7 +1168,7 @@ constexpr int WT = 2;   // targets per thread of the wide kernel
 // lanes; eps: the |d|^2 offset; ne: minus the exponent; half: 0.5 in both lanes.
 // d = X_target - X_source as packed pairs; with COMP (tiles near the block's
 // targets) plus the difference of the low parts of the barycenters,
-// (hi_T - hi_S) + (lo_T - lo_S)
+// (hi_T - hi_S) + (lo_T - lo_S), as in the scalar careful path
 template <bool COMP>
 __device__ __forceinline__ void wide_diff2(unsigned long long tx, unsigned long long ty, unsigned long long tz,
                                            unsigned long long sx, unsigned long long sy, unsigned long long sz,
@@ -1205,28 +1266,28 @@ __device__ __forceinline__ void wide_kernel2(unsigned long long dx_, unsigned lo
 // shared memory of the wide kernel (float4 units): broadcast geometry
 // [NT][3], broadcast low parts [NT][2], source vectors [NT][NW4], Kahan pairs
 // [NP][WT][NT]
-template <int OP, int KC>
+template <int OP>
 constexpr size_t wide_smem_bytes() {
-    using L = OpLayout<OP, KC>;
+    using L = OpLayout<OP, 9>;
     return sizeof(float4) * ((size_t)NT * 3 + 2 * NT + (size_t)NT * L::NW4 + (size_t)(L::NA / 2) * WT * NT);
 }
 
-// chunk of CHW sources of the wide kernel: both targets' kernel values at once,
-// then the accumulations (COMP: compensated d; OWN: the tile may hold the targets)
-template <int OP, int KC, bool COMP, bool OWN, int CHW>
+// chunk of CHW sources of the wide kernel on the packed path: both targets'
+// kernel values at once, then the accumulations (COMP: compensated d)
+template <int OP, bool COMP, int CHW>
 __device__ __forceinline__ void wide_chunk(const float4* sg, const float4* sl, const float4* sw, int c0,
                                            unsigned long long TX, unsigned long long TY, unsigned long long TZ,
                                            unsigned long long LX, unsigned long long LY, unsigned long long LZ,
                                            unsigned long long NXp, unsigned long long NYp, unsigned long long NZp,
                                            unsigned long long EPS, unsigned long long NE, unsigned long long HALF,
-                                           float2 (&pt)[WT][OpLayout<OP, KC>::NA / 2]) {
-    using L = OpLayout<OP, KC>;
+                                           float2 (&pt)[WT][OpLayout<OP, 9>::NA / 2]) {
+    using L = OpLayout<OP, 9>;
     constexpr bool LOW = (OP == TP_OP_A || OP == TP_OP_B0);
     constexpr int NP = L::NA / 2;
     constexpr int NW4 = L::NW4;
     const ulonglong2* sg2 = reinterpret_cast<const ulonglong2*>(sg);
     const ulonglong2* sl2 = reinterpret_cast<const ulonglong2*>(sl);
-#pragma unroll 8
+#pragma unroll 2
     for (int q = 0; q < CHW; ++q) {
         const int jj = c0 + q;
         const ulonglong2 u0 = sg2[3 * jj], u1 = sg2[3 * jj + 1];
@@ -1243,13 +1304,7 @@ __device__ __forceinline__ void wide_chunk(const float4* sg, const float4* sl, c
         } else {
             wide_kernel2<false>(dx, dy, dz, NXp, NYp, NZp, 0ull, 0ull, 0ull, EPS, NE, HALF, HB, H0);
         }
-        float2 hb = upk2(HB), h0 = upk2(H0);
-        if constexpr (OWN) {   // the target itself (d = 0) has no term
-            const float2 ex = upk2(dx), ey = upk2(dy), ez = upk2(dz);
-            const float2 r2 = f2fma(ex, ex, f2fma(ey, ey, f2fma(ez, ez, upk2(EPS))));
-            if (!(r2.x > 2.f * tiny_r2<float>())) hb.x = h0.x = 0.f;
-            if (!(r2.y > 2.f * tiny_r2<float>())) hb.y = h0.y = 0.f;
-        }
+        const float2 hb = upk2(HB), h0 = upk2(H0);
         float2 x2[2 * NW4];
 #pragma unroll
         for (int i = 0; i < NW4; ++i) {
@@ -1280,213 +1335,135 @@ __device__ __forceinline__ void wide_chunk(const float4* sg, const float4* sl, c
     }
 }
 
-// units (256 targets x a tile of 128 sources) are numbered row by row; block b of G
-// takes units [b U / G, (b + 1) U / G)
-__host__ __device__ __forceinline__ long long wide_block(long long u, long long U, long long G) {
-    return ((u + 1) * G - 1) / U;
-}
-
-// resident blocks per SM that the registers and the shared memory are cut for (A with
-// three columns: 3 blocks of 168 registers 643 us at 19,920 faces, 4 of 128 with spills 673;
-// L with three: 5 blocks 278 us, 4 302)
-template <int OP, int KC> struct WideBlocks {
-    static constexpr int NP = OpLayout<OP, KC>::NA / 2;
-    static constexpr int N = NP > 10 ? 2 : NP > 6 ? 3 : NP > 4 ? 4 : 5;
-};
-
-// Equal runs of units to one round of resident blocks: no wave of blocks is left partly
-// empty, and a row of targets meets few blocks, whose partial sums (Kahan pairs in the
-// slot of the block among the row's blocks) the combine adds: 5 slots at 19,920 faces in
-// place of 23 splits, 110 MB of partial sums less per 9-column apply of A. Units of 32
-// sources balance the runs better (130 against 138 us for A with three columns at 7,954
-// faces) but cost the inner loop more than that at 19,920 (955 against 902 with nine).
-template <int OP, int KC, int CHW>
-__global__ void __launch_bounds__(NT, WideBlocks<OP, KC>::N)
+template <int OP, int CHW>
+__global__ void __launch_bounds__(NT, 2)
 k_apply_wide(const float4* __restrict__ fa, const float4* __restrict__ fb, const float4* __restrict__ flo,
              const float4* __restrict__ tbox, const double* __restrict__ center, const float4* __restrict__ Wp,
-             int nf, long long units, float s_exp, float l_exp, float2* __restrict__ part) {
-    using L = OpLayout<OP, KC>;
+             int nf, int tiles_per_split, float s_exp, float l_exp, float2* __restrict__ part) {
+    using L = OpLayout<OP, 9>;
     constexpr bool LOW = (OP == TP_OP_A || OP == TP_OP_B0);
     constexpr int NP = L::NA / 2;
     constexpr int NW4 = L::NW4;
     extern __shared__ float4 wsm[];
     float4* sg = wsm;                        // broadcast geometry: {x,x,y,y} {z,z,nz,nz} {nx,nx,ny,ny}
-    float4* sl = sg + 3 * NT;                // broadcast low parts: {lx,lx,ly,ly} {lz,lz,0,0}
+    float4* sl = sg + 3 * NT;                // broadcast low parts (near tiles): {lx,lx,ly,ly} {lz,lz,0,0}
     float4* sw = sl + 2 * NT;                // source vectors X
     float4* kah = sw + NT * NW4;             // Kahan pairs {s.x, s.y, c.x, c.y}
+    __shared__ float sbox[6];
     const int tid = threadIdx.x;
-    const int ntiles = (nf + NT - 1) / NT;
+    float tx[WT], ty[WT], tz[WT], nx[WT], ny[WT], nz[WT], lx[WT], ly[WT], lz[WT];
+    int tg[WT];
+    float bl[3] = {3e38f, 3e38f, 3e38f}, bh[3] = {-3e38f, -3e38f, -3e38f};
+#pragma unroll
+    for (int j = 0; j < WT; ++j) {
+        const int t = blockIdx.x * NT * WT + j * NT + tid;
+        tg[j] = t;
+        tx[j] = ty[j] = tz[j] = nx[j] = ny[j] = nz[j] = 0.f;
+        lx[j] = ly[j] = lz[j] = 0.f;
+        if (t < nf) {
+            const float4 A = fa[t];
+            tx[j] = A.x; ty[j] = A.y; tz[j] = A.z;
+            if (LOW) {
+                const float4 B = fb[t];
+                nx[j] = B.x; ny[j] = B.y; nz[j] = B.z;
+            }
+            const float4 Lo = flo[t];
+            lx[j] = Lo.x; ly[j] = Lo.y; lz[j] = Lo.z;
+            bl[0] = fminf(bl[0], A.x); bl[1] = fminf(bl[1], A.y); bl[2] = fminf(bl[2], A.z);
+            bh[0] = fmaxf(bh[0], A.x); bh[1] = fmaxf(bh[1], A.y); bh[2] = fmaxf(bh[2], A.z);
+        }
+    }
+    block_box(bl[0], bl[1], bl[2], bh[0], bh[1], bh[2], sbox);
     const float thr2 = (float)center[3];
+    const unsigned long long TX = pk2(tx[0], tx[1]), TY = pk2(ty[0], ty[1]), TZ = pk2(tz[0], tz[1]);
+    const unsigned long long LX = pk2(lx[0], lx[1]), LY = pk2(ly[0], ly[1]), LZ = pk2(lz[0], lz[1]);
+    const unsigned long long NXp = pk2(nx[0], nx[1]), NYp = pk2(ny[0], ny[1]), NZp = pk2(nz[0], nz[1]);
     const unsigned long long EPS = pk2(tiny_r2<float>(), tiny_r2<float>());
     const float nexp = OP == TP_OP_L ? -l_exp : -s_exp;
     const unsigned long long NE = pk2(nexp, nexp), HALF = pk2(0.5f, 0.5f);
-    const long long u1 = units * (blockIdx.x + 1) / gridDim.x;
-    for (long long u = units * blockIdx.x / gridDim.x; u < u1;) {
-        const int row = (int)(u / ntiles);
-        const long long uend = min(u1, (long long)(row + 1) * ntiles);
-        float tx[WT], ty[WT], tz[WT], nx[WT], ny[WT], nz[WT], lx[WT], ly[WT], lz[WT];
-        float bl[3] = {3e38f, 3e38f, 3e38f}, bh[3] = {-3e38f, -3e38f, -3e38f};
 #pragma unroll
-        for (int j = 0; j < WT; ++j) {
-            const int t = row * NT * WT + j * NT + tid;
-            tx[j] = ty[j] = tz[j] = nx[j] = ny[j] = nz[j] = 0.f;
-            lx[j] = ly[j] = lz[j] = 0.f;
-            if (t < nf) {
-                const float4 A = fa[t];
-                tx[j] = A.x; ty[j] = A.y; tz[j] = A.z;
-                if (LOW) {
-                    const float4 B = fb[t];
-                    nx[j] = B.x; ny[j] = B.y; nz[j] = B.z;
-                }
-                const float4 Lo = flo[t];
-                lx[j] = Lo.x; ly[j] = Lo.y; lz[j] = Lo.z;
-                bl[0] = fminf(bl[0], A.x); bl[1] = fminf(bl[1], A.y); bl[2] = fminf(bl[2], A.z);
-                bh[0] = fmaxf(bh[0], A.x); bh[1] = fmaxf(bh[1], A.y); bh[2] = fmaxf(bh[2], A.z);
-            }
-        }
-        for (int o = 16; o > 0; o >>= 1)   // the box of the warp's targets
-            for (int c = 0; c < 3; ++c) {
-                bl[c] = fminf(bl[c], __shfl_xor_sync(0xffffffffu, bl[c], o));
-                bh[c] = fmaxf(bh[c], __shfl_xor_sync(0xffffffffu, bh[c], o));
-            }
-        const float sbox[6] = {bl[0], bl[1], bl[2], bh[0], bh[1], bh[2]};
-        const unsigned long long TX = pk2(tx[0], tx[1]), TY = pk2(ty[0], ty[1]), TZ = pk2(tz[0], tz[1]);
-        const unsigned long long LX = pk2(lx[0], lx[1]), LY = pk2(ly[0], ly[1]), LZ = pk2(lz[0], lz[1]);
-        const unsigned long long NXp = pk2(nx[0], nx[1]), NYp = pk2(ny[0], ny[1]), NZp = pk2(nz[0], nz[1]);
-#pragma unroll
-        for (int i = 0; i < NP * WT; ++i) kah[i * NT + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (; u < uend; ++u) {
-            const int tile = (int)(u - (long long)row * ntiles);
-            const bool near = tile_near(tbox, tile, sbox, thr2);
-            const int src = tile * NT + tid;
-            __syncthreads();
-            {
-                // sources past the end sit far away with zero vectors: finite zero terms
-                const float4 A = src < nf ? fa[src] : make_float4(1e18f, 0.f, 0.f, 0.f);
-                const float4 B = (LOW && src < nf) ? fb[src] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < NP * WT; ++i) kah[i * NT + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int ntiles = (nf + NT - 1) / NT;
+    const int k0 = blockIdx.y * tiles_per_split;
+    const int k1 = min(k0 + tiles_per_split, ntiles);
+    for (int tile = k0; tile < k1; ++tile) {
+        const bool diag = tile >= (int)blockIdx.x * WT && tile < ((int)blockIdx.x + 1) * WT;
+        const bool near = tile_near(tbox, tile, sbox, thr2);
+        const int src = tile * NT + tid;
+        __syncthreads();
+        {
+            // sources past the end sit far away with zero vectors: finite zero terms
+            const float4 A = src < nf ? fa[src] : make_float4(1e18f, 0.f, 0.f, 0.f);
+            const float4 B = (LOW && src < nf) ? fb[src] : make_float4(0.f, 0.f, 0.f, 0.f);
+            sg[3 * tid] = make_float4(A.x, A.x, A.y, A.y);
+            sg[3 * tid + 1] = make_float4(A.z, A.z, B.z, B.z);
+            sg[3 * tid + 2] = make_float4(B.x, B.x, B.y, B.y);
+            if (near || diag) {
                 const float4 l = src < nf ? flo[src] : make_float4(0.f, 0.f, 0.f, 0.f);
-                sg[3 * tid] = make_float4(A.x, A.x, A.y, A.y);
-                sg[3 * tid + 1] = make_float4(A.z, A.z, B.z, B.z);
-                sg[3 * tid + 2] = make_float4(B.x, B.x, B.y, B.y);
                 sl[2 * tid] = make_float4(l.x, l.x, l.y, l.y);
                 sl[2 * tid + 1] = make_float4(l.z, l.z, 0.f, 0.f);
             }
-            for (int i = tid; i < NT * NW4; i += NT) {
-                const int f = tile * NT + i / NW4;
-                sw[i] = f < nf ? Wp[(size_t)tile * NT * NW4 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            __syncthreads();
+        }
+        for (int i = tid; i < NT * NW4; i += NT) {
+            const int f = tile * NT + i / NW4;
+            sw[i] = f < nf ? Wp[(size_t)tile * NT * NW4 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        __syncthreads();
+        for (int c = 0; c < NT; c += CHW) {
             float2 pt[WT][NP];
 #pragma unroll
             for (int j = 0; j < WT; ++j)
 #pragma unroll
                 for (int i = 0; i < NP; ++i) pt[j][i] = make_float2(0.f, 0.f);
-            for (int c = 0; c < NT; c += CHW) {
-                if (tile / WT == row)
-                    wide_chunk<OP, KC, true, true, CHW>(sg, sl, sw, c, TX, TY, TZ, LX, LY, LZ, NXp, NYp, NZp, EPS, NE, HALF,
-                                                   pt);
-                else if (near)
-                    wide_chunk<OP, KC, true, false, CHW>(sg, sl, sw, c, TX, TY, TZ, LX, LY, LZ, NXp, NYp, NZp, EPS, NE,
-                                                    HALF, pt);
-                else
-                    wide_chunk<OP, KC, false, false, CHW>(sg, sl, sw, c, TX, TY, TZ, LX, LY, LZ, NXp, NYp, NZp, EPS, NE,
-                                                     HALF, pt);
-                // chunk sums into the Kahan pairs in shared memory
+            if (diag) {
+                // tiles holding the block's own targets: scalar careful path with
+                // the self-pair test
+                for (int q = 0; q < CHW; ++q) {
+                    const int jj = c + q;
+                    const float4 g0 = sg[3 * jj], g1 = sg[3 * jj + 1], g2 = sg[3 * jj + 2];
+                    const float4 l0 = sl[2 * jj], l1 = sl[2 * jj + 1];
+                    float2 wv[2 * NW4];
 #pragma unroll
-                for (int j = 0; j < WT; ++j)
-#pragma unroll
-                    for (int i = 0; i < NP; ++i) {
-                        float4& k = kah[(i * WT + j) * NT + tid];
-                        const float4 kv = k;
-                        const float2 s = make_float2(kv.x, kv.y), cc = make_float2(kv.z, kv.w);
-                        const float2 y = psub(pt[j][i], cc);
-                        const float2 t = padd(s, y);
-                        const float2 cn = psub(psub(t, s), y);
-                        k = make_float4(t.x, t.y, cn.x, cn.y);
-                        pt[j][i] = make_float2(0.f, 0.f);
+                    for (int i = 0; i < NW4; ++i) {
+                        const float4 x = sw[jj * NW4 + i];
+                        wv[2 * i] = make_float2(x.x, x.y);
+                        wv[2 * i + 1] = make_float2(x.z, x.w);
                     }
+#pragma unroll
+                    for (int j = 0; j < WT; ++j)
+                        apply_term<float, OP, true, 9>((tx[j] - g0.x) + (lx[j] - l0.x), (ty[j] - g0.z) + (ly[j] - l0.z),
+                                                       (tz[j] - g1.x) + (lz[j] - l1.x), nx[j], ny[j], nz[j], g2.x,
+                                                       g2.z, g1.z, wv, s_exp, l_exp, pt[j]);
+                }
+            } else if (near) {
+                wide_chunk<OP, true, CHW>(sg, sl, sw, c, TX, TY, TZ, LX, LY, LZ, NXp, NYp, NZp, EPS, NE, HALF, pt);
+            } else {
+                wide_chunk<OP, false, CHW>(sg, sl, sw, c, TX, TY, TZ, LX, LY, LZ, NXp, NYp, NZp, EPS, NE, HALF, pt);
             }
-        }
-        const long long slot = (long long)blockIdx.x - wide_block((long long)row * ntiles, units, gridDim.x);
+            // chunk sums into the Kahan pairs in shared memory
 #pragma unroll
-        for (int j = 0; j < WT; ++j) {
-            const int t = row * NT * WT + j * NT + tid;
-            if (t < nf)
+            for (int j = 0; j < WT; ++j)
 #pragma unroll
-                for (int a = 0; a < L::NA; ++a) {
-                    const float4 kv = kah[((a / 2) * WT + j) * NT + tid];
-                    part[((size_t)slot * L::NA + a) * nf + t] =
-                        (a & 1) ? make_float2(kv.y, kv.w) : make_float2(kv.x, kv.z);
+                for (int i = 0; i < NP; ++i) {
+                    float4& k = kah[(i * WT + j) * NT + tid];
+                    const float4 kv = k;
+                    const float2 s = make_float2(kv.x, kv.y), cc = make_float2(kv.z, kv.w);
+                    const float2 y = psub(pt[j][i], cc);
+                    const float2 t = padd(s, y);
+                    const float2 cn = psub(psub(t, s), y);
+                    k = make_float4(t.x, t.y, cn.x, cn.y);
                 }
         }
     }
-}
-
-// k_apply_combine for the wide kernel's slots: the slots' Kahan pairs (sum s - c) in slot
-// order as unevaluated FP32 pairs (about 48 bits; FP64 additions would take longer than
-// the reads), then as there. Lanes take consecutive faces.
-template <int OP, int KC>
-__global__ void __launch_bounds__(32 * (KC + 1))
-k_wide_combine(const float2* __restrict__ part, int nf, long long ntiles, long long units, long long G,
-               const d4* __restrict__ f64a, const double* __restrict__ fgrad, const double* __restrict__ W64, int k,
-               int col0, double* __restrict__ corner) {
-    using L = OpLayout<OP, KC>;
-    __shared__ double s_hi[32], s_lo[32];
-    const int fl = threadIdx.x, c = threadIdx.y, S = blockIdx.x * 32 + fl;
-    const long long row = blockIdx.x * 32 / (NT * WT);   // 32 divides a row: one row per block
-    const int slots =
-        (int)(wide_block((row + 1) * ntiles - 1, units, G) - wide_block(row * ntiles, units, G)) + 1;
-    const bool has = S < nf;
-    struct Sum {   // unevaluated pair: hi takes the slots' sums, lo the exact rounding errors and the -c
-        float hi = 0.f, lo = 0.f;
-        __device__ __forceinline__ void add(float2 v) {
-            const float t = hi + v.x, z = t - hi;
-            lo += ((hi - (t - z)) + (v.x - z)) - v.y;
-            hi = t;
-        }
-        __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-    };
-    const double a = has ? f64a[S].w : 1.0;
-    Sum v[4];
-    const bool area = has && c == KC, mine = has && c < KC && col0 + c < k;
-    if (area || mine) {
-        // the area sums, or the column's three high-order sums and its low-order one
-        int at[4];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) at[q] = area ? 0 : 1 + q * KC + c;
-        at[3] = L::NH + (area ? 0 : 1 + c);
-#pragma unroll 4
-        for (int s = 0; s < slots; ++s) {
-            const float2* ps = part + (size_t)s * L::NA * nf + S;
-            if (L::HIGH) {
+    for (int j = 0; j < WT; ++j)
+        if (tg[j] < nf)
 #pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (q == 0 || !area) v[q].add(ps[(size_t)at[q] * nf]);
+            for (int a = 0; a < L::NA; ++a) {
+                const float4 kv = kah[((a / 2) * WT + j) * NT + tid];
+                part[((size_t)blockIdx.y * L::NA + a) * nf + tg[j]] =
+                    (a & 1) ? make_float2(kv.y, kv.w) : make_float2(kv.x, kv.z);
             }
-            if (L::USEU) v[3].add(ps[(size_t)at[3] * nf]);
-        }
-    }
-    if (area) {
-        const double ia = 1.0 / a;
-        s_hi[fl] = v[0].value() * ia;
-        s_lo[fl] = v[3].value() * ia;
-    }
-    __syncthreads();
-    if (!mine) return;
-    const double* W = W64 + 4 * KC * (size_t)S;
-    double zV[3], zU = 0.0;
-    if (L::HIGH)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) zV[q] = s_hi[fl] * W[q * KC + c] - v[q].value();
-    if (L::USEU) zU = (s_lo[fl] * W[3 * KC + c] - v[3].value()) * (1.0 / 3.0);
-    const double* gr = fgrad + 9 * (size_t)S;
-    const double a2 = 2.0 * a;
-#pragma unroll
-    for (int cr = 0; cr < 3; ++cr) {
-        double g = zU;
-        if (L::HIGH) g += gr[3 * cr] * zV[0] + gr[3 * cr + 1] * zV[1] + gr[3 * cr + 2] * zV[2];
-        corner[((size_t)S * 3 + cr) * k + col0 + c] = a2 * g;
-    }
 }
 
 // sums over the source splits of the wide kernel's partial Kahan pairs, one
@@ -1639,20 +1616,27 @@ static RootPow root_plan(double p, bool op_l) {
     return r;
 }
 
-template <int OP, int KC>
+template <typename T, int OP, int KC>
 static int launch_apply_op(tp_mesh* m, const tp_params* p, const double* v, int k, double* y,
                            cudaStream_t st) {
+    using V4 = typename V4T<T>::type;
     using L = OpLayout<OP, KC>;
     const int nf = m->nf;
-    const Grid g = fp64_grid(make_grid(nf, nf, 1, resident_per_sm((const void*)k_apply<OP, KC>, NT)), nf);
+    const double s = 2.0 - 2.0 / p->p;       // Sobolev order, §2.3
+    const double l_exp = 3.0 - s;            // |d|^{-(2 sigma + 2)} = r2^{-(sigma+1)}, sigma = 2 - s
+    constexpr int TT = (sizeof(T) == 4 && KC == 3) ? 2 : 1;
+    Grid g = make_grid(nf, nf, TT, resident_per_sm((const void*)k_apply<T, OP, TT, KC>, NT));
+    if (sizeof(T) == 8) g = fp64_grid(g, nf);
     TP_TRY(ensure(m->part, sizeof(double) * (size_t)g.nsplit * L::NA * nf));
     TP_TRY(ensure(m->wv64, sizeof(double) * 4 * KC * (size_t)nf));
-    TP_TRY(ensure(m->wv32, sizeof(d4) * L::NW4 * (size_t)nf));
+    TP_TRY(ensure(m->wv32, sizeof(V4) * L::NW4 * (size_t)nf));
     TP_TRY(ensure(m->corner, sizeof(double) * 3 * (size_t)nf * k));
+    const V4* fa = (const V4*)(sizeof(T) == 4 ? m->f32a.ptr : m->f64a.ptr);
+    const V4* fb = (const V4*)(sizeof(T) == 4 ? m->f32b.ptr : m->f64b.ptr);
     for (int col0 = 0; col0 < k; col0 += KC) {
-        k_face_W<double, KC><<<(nf * ((KC + 2) / 3) + 255) / 256, 256, 0, st>>>(v, k, col0, m->faces.as<int>(), nf,
+        k_face_W<T, KC><<<(nf * ((KC + 2) / 3) + 255) / 256, 256, 0, st>>>(v, k, col0, m->faces.as<int>(), nf,
                                                           m->f64a.as<d4>(), m->fgrad.as<double>(), OP,
-                                                          m->wv64.as<double>(), m->wv32.as<d4>(), L::NW4);
+                                                          m->wv64.as<double>(), m->wv32.as<V4>(), L::NW4);
         TP_LAUNCH_CHECK();
         dim3 grid(g.bx, g.nsplit);
         {
@@ -1662,9 +1646,10 @@ static int launch_apply_op(tp_mesh* m, const tp_params* p, const double* v, int 
                               : OP == TP_OP_B0 ? PK_APPLY_B0 : PK_APPLY_L;
             ProfScope ps(m, key, units, st);
             m->prof.cols[key] += KC;
-            k_apply<OP, KC><<<grid, NT, two_resident(k_apply<OP, KC>), st>>>(
-                m->f64a.as<d4>(), m->f64b.as<d4>(), m->wv32.as<d4>(), nf, g.tiles_per_split, m->part.as<double>(),
-                root_plan(p->p, OP == TP_OP_L));
+            k_apply<T, OP, TT, KC><<<grid, NT, sizeof(T) == 8 ? two_resident(k_apply<T, OP, TT, KC>) : 0, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
+                                                        m->center.as<double>(), m->wv32.as<V4>(), nf,
+                                                        g.tiles_per_split, T(s), T(l_exp), m->part.as<double>(),
+                                                        root_plan(p->p, OP == TP_OP_L));
         }
         TP_LAUNCH_CHECK();
         k_apply_combine<OP, KC><<<(nf + 31) / 32, dim3(32, KC + 1), 0, st>>>(m->part.as<double>(), g.nsplit, nf,
@@ -1676,6 +1661,7 @@ static int launch_apply_op(tp_mesh* m, const tp_params* p, const double* v, int 
     return corners_to_vertices(m, m->corner.as<double>(), k, y, st);
 }
 
+// FP32, 9 columns: the two-targets-per-thread kernel (k_apply_wide)
 // ---------------------------------------------------------------------------
 // 9-column A apply with the accumulation on tcgen05 tensor cores
 // ---------------------------------------------------------------------------
@@ -2178,89 +2164,81 @@ int apply_tc_error(tp_mesh* m, int* gave_up, cudaStream_t st) {
     return TP_OK;
 }
 
-template <int OP, int KC>
+template <int OP>
 static int launch_apply_wide(tp_mesh* m, const tp_params* p, const double* v, int k, double* y, cudaStream_t st) {
-    using L = OpLayout<OP, KC>;
-    // sources per FP32 chunk sum before the Kahan update: whole tiles where many
-    // accumulators are flushed, half and quarter tiles where few are
-    constexpr int CHW = L::NA > 20 ? 128 : KC > 3 ? 64 : 32;
+    using L = OpLayout<OP, 9>;
+    // sources per FP32 chunk sum before the Kahan update: whole tiles for the
+    // operators with the high-order part (many accumulators per flush), half
+    // tiles for the others
+    constexpr int CHW = (OP == TP_OP_A || OP == TP_OP_B) ? 128 : 64;
     const int nf = m->nf;
     const double s = 2.0 - 2.0 / p->p;
     const double l_exp = 3.0 - s;
-    const size_t smem = wide_smem_bytes<OP, KC>();
-    const int per_sm = resident_per_sm((const void*)k_apply_wide<OP, KC, CHW>, NT, smem);
+    const size_t smem = wide_smem_bytes<OP>();
+    const int per_sm = resident_per_sm((const void*)k_apply_wide<OP, CHW>, NT, smem);
     if (per_sm < 1) return fail(TP_ERR_CUDA, "k_apply_wide: shared memory per block not available");
-    const long long ntiles = (nf + NT - 1) / NT, rows = (nf + NT * WT - 1) / (NT * WT), units = ntiles * rows;
-    const long long G = std::min<long long>(units, (long long)per_sm * sm_count());
-    long long slots = 1;   // most blocks that share a row
-    for (long long r = 0; r < rows; ++r)
-        slots = std::max(slots, wide_block((r + 1) * ntiles - 1, units, G) - wide_block(r * ntiles, units, G) + 1);
-    TP_TRY(ensure(m->part, sizeof(float2) * (size_t)slots * L::NA * nf));
-    TP_TRY(ensure(m->wv64, sizeof(double) * 4 * KC * (size_t)nf));
+    Grid g = make_grid(nf, nf, WT, per_sm);
+    TP_TRY(ensure(m->part, sizeof(float2) * (size_t)g.nsplit * L::NA * nf + sizeof(double) * L::NA * (size_t)nf));
+    TP_TRY(ensure(m->wv64, sizeof(double) * 4 * 9 * (size_t)nf));
     TP_TRY(ensure(m->wv32, sizeof(float4) * L::NW4 * (size_t)nf));
     TP_TRY(ensure(m->corner, sizeof(double) * 3 * (size_t)nf * k));
     const float4* fa = m->f32a.as<float4>();
     const float4* fb = m->f32b.as<float4>();
-    for (int col0 = 0; col0 < k; col0 += KC) {
-        k_face_W<float, KC><<<(nf * (KC / 3) + 255) / 256, 256, 0, st>>>(v, k, col0, m->faces.as<int>(), nf,
-                                                                        m->f64a.as<d4>(), m->fgrad.as<double>(), OP,
-                                                                        m->wv64.as<double>(), m->wv32.as<float4>(),
-                                                                        L::NW4);
+    for (int col0 = 0; col0 < k; col0 += 9) {
+        k_face_W<float, 9><<<(nf * 3 + 255) / 256, 256, 0, st>>>(v, k, col0, m->faces.as<int>(), nf, m->f64a.as<d4>(),
+                                                             m->fgrad.as<double>(), OP, m->wv64.as<double>(),
+                                                             m->wv32.as<float4>(), L::NW4);
         TP_LAUNCH_CHECK();
+        dim3 grid(g.bx, g.nsplit);
         {
-            const double pairs = (double)nf * (nf - 1);
-            m->pairs += pairs;
+            const double units = (double)nf * (nf - 1);
+            m->pairs += units;
             constexpr int key = OP == TP_OP_A ? PK_APPLY_A : OP == TP_OP_B ? PK_APPLY_B
                               : OP == TP_OP_B0 ? PK_APPLY_B0 : PK_APPLY_L;
-            ProfScope ps(m, key, pairs, st);
-            m->prof.cols[key] += KC;
-            k_apply_wide<OP, KC, CHW><<<(unsigned)G, NT, smem, st>>>(fa, fb, m->f32c.as<float4>(),
-                                                                    m->tilebox.as<float4>(), m->center.as<double>(),
-                                                                    m->wv32.as<float4>(), nf, units, (float)s,
-                                                                    (float)l_exp, m->part.as<float2>());
+            ProfScope ps(m, key, units, st);
+            m->prof.cols[key] += 9;
+            k_apply_wide<OP, CHW><<<grid, NT, smem, st>>>(fa, fb, m->f32c.as<float4>(), m->tilebox.as<float4>(),
+                                                          m->center.as<double>(), m->wv32.as<float4>(), nf,
+                                                          g.tiles_per_split, (float)s, (float)l_exp,
+                                                          m->part.as<float2>());
         }
         TP_LAUNCH_CHECK();
-        k_wide_combine<OP, KC><<<(nf + 31) / 32, dim3(32, KC + 1), 0, st>>>(
-            m->part.as<float2>(), nf, ntiles, units, G, m->f64a.as<d4>(), m->fgrad.as<double>(), m->wv64.as<double>(), k,
-            col0, m->corner.as<double>());
+        double* sums = reinterpret_cast<double*>(m->part.as<float2>() + (size_t)g.nsplit * L::NA * nf);
+        k_split_sum2<<<(unsigned)(((size_t)L::NA * nf + 255) / 256), 256, 0, st>>>(m->part.as<float2>(), g.nsplit,
+                                                                                L::NA, nf, sums);
+        TP_LAUNCH_CHECK();
+        k_apply_combine2<OP, 9><<<(nf + SC_FACES - 1) / SC_FACES, SC_FACES * 9, 0, st>>>(
+            sums, nf, m->f64a.as<d4>(), m->fgrad.as<double>(), m->wv64.as<double>(), k, col0, m->corner.as<double>());
         TP_LAUNCH_CHECK();
     }
     return corners_to_vertices(m, m->corner.as<double>(), k, y, st);
 }
 
-// three columns a pass, six or nine: the columns of a pass share the kernel values (A at
-// 19,920 faces: 579, 774 and 902 us, so a pass that fits the columns beats a padded wider one
-// and two narrower ones)
-template <int OP>
-static int launch_apply_f32(tp_mesh* m, const tp_params* p, const double* v, int k, double* y, cudaStream_t st) {
-    return k <= 3   ? launch_apply_wide<OP, 3>(m, p, v, k, y, st)
-           : k <= 6 ? launch_apply_wide<OP, 6>(m, p, v, k, y, st)
-                    : launch_apply_wide<OP, 9>(m, p, v, k, y, st);
-}
-
 template <typename T>
 static int launch_apply(tp_mesh* m, const tp_params* p, int op, const double* v, int k, double* y,
                         cudaStream_t st) {
+    // 9 columns in one pass share the kernel evaluation; up to 3 columns
+    // take the lighter 3-column kernel
     const bool wide = k > 3;
-    if constexpr (sizeof(T) == 4) {
+    if (sizeof(T) == 4 && wide) {
         switch (op) {
-            case TP_OP_A: return p->tensor_cores && wide ? launch_apply_tc(m, p, v, k, y, st)
-                                                         : launch_apply_f32<TP_OP_A>(m, p, v, k, y, st);
-            case TP_OP_B: return launch_apply_f32<TP_OP_B>(m, p, v, k, y, st);
-            case TP_OP_B0: return launch_apply_f32<TP_OP_B0>(m, p, v, k, y, st);
-            case TP_OP_L: return launch_apply_f32<TP_OP_L>(m, p, v, k, y, st);
+            case TP_OP_A: return p->tensor_cores ? launch_apply_tc(m, p, v, k, y, st)
+                                                 : launch_apply_wide<TP_OP_A>(m, p, v, k, y, st);
+            case TP_OP_B: return launch_apply_wide<TP_OP_B>(m, p, v, k, y, st);
+            case TP_OP_B0: return launch_apply_wide<TP_OP_B0>(m, p, v, k, y, st);
+            case TP_OP_L: return launch_apply_wide<TP_OP_L>(m, p, v, k, y, st);
         }
-    } else {
-        switch (op) {
-            case TP_OP_A: return wide ? launch_apply_op<TP_OP_A, 9>(m, p, v, k, y, st)
-                                      : launch_apply_op<TP_OP_A, 3>(m, p, v, k, y, st);
-            case TP_OP_B: return wide ? launch_apply_op<TP_OP_B, 9>(m, p, v, k, y, st)
-                                      : launch_apply_op<TP_OP_B, 3>(m, p, v, k, y, st);
-            case TP_OP_B0: return wide ? launch_apply_op<TP_OP_B0, 9>(m, p, v, k, y, st)
-                                       : launch_apply_op<TP_OP_B0, 3>(m, p, v, k, y, st);
-            case TP_OP_L: return wide ? launch_apply_op<TP_OP_L, 9>(m, p, v, k, y, st)
-                                      : launch_apply_op<TP_OP_L, 3>(m, p, v, k, y, st);
-        }
+        return fail(TP_ERR_INVALID_ARG, "unknown operator");
+    }
+    switch (op) {
+        case TP_OP_A: return wide ? launch_apply_op<T, TP_OP_A, 9>(m, p, v, k, y, st)
+                                  : launch_apply_op<T, TP_OP_A, 3>(m, p, v, k, y, st);
+        case TP_OP_B: return wide ? launch_apply_op<T, TP_OP_B, 9>(m, p, v, k, y, st)
+                                  : launch_apply_op<T, TP_OP_B, 3>(m, p, v, k, y, st);
+        case TP_OP_B0: return wide ? launch_apply_op<T, TP_OP_B0, 9>(m, p, v, k, y, st)
+                                   : launch_apply_op<T, TP_OP_B0, 3>(m, p, v, k, y, st);
+        case TP_OP_L: return wide ? launch_apply_op<T, TP_OP_L, 9>(m, p, v, k, y, st)
+                                  : launch_apply_op<T, TP_OP_L, 3>(m, p, v, k, y, st);
     }
     return fail(TP_ERR_INVALID_ARG, "unknown operator");
 }
