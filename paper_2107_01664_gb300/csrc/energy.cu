@@ -112,9 +112,9 @@ struct Tile {
 
 __device__ __forceinline__ void stage(Tile& t, const float4* __restrict__ fa, const float4* __restrict__ fb,
                                       const float4* __restrict__ fl, int src, int nf, bool low) {
-    // sources past the end: zero area and normal (all their terms are zero)
+    // sources past the end: far away, zero area and normal (all their terms are zero)
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 A = src < nf ? fa[src] : z, N = src < nf ? fb[src] : z;
+    const float4 A = src < nf ? fa[src] : make_float4(PAD_X, 0.f, 0.f, 0.f), N = src < nf ? fb[src] : z;
     ulonglong2* g = t.g[threadIdx.x];
     g[0] = make_ulonglong2(pk(A.x, A.x), pk(A.y, A.y));
     g[1] = make_ulonglong2(pk(A.z, A.z), pk(A.w, A.w));

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(NA_T) k_na_pairs(NoAllocScratch* sc, int nf, i
     for (int tile = k0; tile < k1; ++tile) {
         const int src = tile * NA_T + threadIdx.x;
         __syncthreads();
-        sx[threadIdx.x] = src < nf ? sc->xa[src] : make_float4(0.f, 0.f, 0.f, 0.f);
+        sx[threadIdx.x] = src < nf ? sc->xa[src] : make_float4(tp::PAD_X, 0.f, 0.f, 0.f);
         sl[threadIdx.x] = src < nf ? sc->xl[src] : make_float4(0.f, 0.f, 0.f, 0.f);
         __syncthreads();
         for (int c = 0; c < NA_T; c += NA_CH) {

@@ -37,7 +37,6 @@ namespace {
 
 constexpr int NT = 128;  // threads per block = obstacle faces per shared-memory tile
 constexpr int CH = 32;   // sources per FP32 run before the compensated add
-constexpr float PAD_X = 1e18f;   // x of the padding sources of the last tile (area 0, far away)
 
 template <typename T> struct V4O;
 template <> struct V4O<float> { using type = float4; };

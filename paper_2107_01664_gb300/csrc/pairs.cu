@@ -31,6 +31,12 @@ template <> struct V4T<double> { using type = d4; };
 template <typename T> __device__ __forceinline__ typename V4T<T>::type v4zero();
 template <> __device__ __forceinline__ float4 v4zero<float>() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 template <> __device__ __forceinline__ d4 v4zero<double>() { return d4{0.0, 0.0, 0.0, 0.0}; }
+// barycenter and area of a source past the end of the mesh. FP64 stays at the origin:
+// its kernel values are finite at any distance above 1e-50, and root_pow keeps to its
+// fast range
+template <typename T> __device__ __forceinline__ typename V4T<T>::type v4pad();
+template <> __device__ __forceinline__ float4 v4pad<float>() { return make_float4(PAD_X, 0.f, 0.f, 0.f); }
+template <> __device__ __forceinline__ d4 v4pad<double>() { return v4zero<double>(); }
 
 // ---- elementary functions (FP32: single MUFU instructions) --------------
 
@@ -457,7 +463,7 @@ k_energy(const typename V4T<T>::type* __restrict__ fa, const typename V4T<T>::ty
         const bool near = F32 && tile_near(tbox, tile, sbox, thr2);
         int src = tile * NT + threadIdx.x;
         __syncthreads();
-        const V4 sv = src < nf ? fa[src] : v4zero<T>();   // zero area pads the tail
+        const V4 sv = src < nf ? fa[src] : v4pad<T>();
         sh[threadIdx.x] = sv;
         if constexpr (PACK) {
             shp[2 * threadIdx.x] = make_ulonglong2(pk2((float)sv.x, (float)sv.x), pk2((float)sv.y, (float)sv.y));
@@ -661,7 +667,7 @@ k_diff(const typename V4T<T>::type* __restrict__ fa, const typename V4T<T>::type
         const bool near = F32 && tile_near(tbox, tile, sbox, thr2);
         int src = tile * NT + threadIdx.x;
         __syncthreads();
-        sa[threadIdx.x] = src < nf ? fa[src] : v4zero<T>();
+        sa[threadIdx.x] = src < nf ? fa[src] : v4pad<T>();
         sb[threadIdx.x] = src < nf ? fb[src] : v4zero<T>();
         if (near) shl[threadIdx.x] = src < nf ? flo[src] : make_float4(0.f, 0.f, 0.f, 0.f);
         __syncthreads();
@@ -1073,7 +1079,7 @@ k_apply(const typename V4T<T>::type* __restrict__ fa, const typename V4T<T>::typ
         const bool near = F32 && tile_near(tbox, tile, sbox, thr2);
         int src = tile * NT + threadIdx.x;
         __syncthreads();
-        sa[threadIdx.x] = src < nf ? fa[src] : v4zero<T>();
+        sa[threadIdx.x] = src < nf ? fa[src] : v4pad<T>();
         if (LOW) sb[threadIdx.x] = src < nf ? fb[src] : v4zero<T>();
         if (near) shl[threadIdx.x] = src < nf ? flo[src] : make_float4(0.f, 0.f, 0.f, 0.f);
         for (int i = threadIdx.x; i < NT * L::NW4; i += NT) {
@@ -1393,7 +1399,7 @@ k_apply_wide(const float4* __restrict__ fa, const float4* __restrict__ fb, const
         __syncthreads();
         {
             // sources past the end sit far away with zero vectors: finite zero terms
-            const float4 A = src < nf ? fa[src] : make_float4(1e18f, 0.f, 0.f, 0.f);
+            const float4 A = src < nf ? fa[src] : v4pad<float>();
             const float4 B = (LOW && src < nf) ? fb[src] : make_float4(0.f, 0.f, 0.f, 0.f);
             sg[3 * tid] = make_float4(A.x, A.x, A.y, A.y);
             sg[3 * tid + 1] = make_float4(A.z, A.z, B.z, B.z);

@@ -70,6 +70,11 @@ struct alignas(32) d4 {
 // number of SMs of the current device (cached per device)
 int sm_count();
 
+// x of the sources that pad a last tile (y = z = 0, zero area, normal and vector):
+// far away, so that every kernel value at them is finite and zero times it is zero. At
+// the origin, the frame's centre, a face within 4e-7 of it would make |d|^-6 infinite.
+constexpr float PAD_X = 1e18f;
+
 // ---------------------------------------------------------------------------
 // FP64 divisions and roots in few operations
 // ---------------------------------------------------------------------------
