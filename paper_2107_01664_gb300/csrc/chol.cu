@@ -850,8 +850,11 @@ __device__ bool wait_until(const unsigned* p, unsigned target, bool at_least, Ch
 // reset; the last block to finish the residual resets the counters and
 // advances the epoch.
 // WIDE: the tree has fronts of more than 256 rows (their matvecs, and vectors of the
-// children read in place). Without those paths the kernel is 1 to 4 us shorter a
-// sweep on meshes of 1,000 to 10,000 vertices.
+// children read in place), or the sweep runs in three launches. Without those paths
+// the kernel is 1 to 4 us shorter a sweep on meshes of 1,000 to 10,000 vertices, and
+// with the tickets' range known it needs no spills at nine columns (1,890 vertices, a
+// solve of two sweeps on three columns, medians over ten meshes: 173 -> 169 us, 165 us
+// before there was a WIDE variant; where the allocations land moves one mesh by 4%).
 template <int K, bool WIDE>
 __global__ void __launch_bounds__(CHS_T)
 k_chol_sweep(SweepArgs A) {
@@ -864,16 +867,17 @@ k_chol_sweep(SweepArgs A) {
     __shared__ double s_red[CHS_T];
     const unsigned ep = *(volatile unsigned*)&ctl->epoch + 1;
     const int nn = A.nn, tid = threadIdx.x;
-    unsigned* ticket = &ctl->ticket[A.phase];
-    if (tid == 0) s_tk = A.t0 + (int)atomicAdd(ticket, 1u);
+    unsigned* ticket = &ctl->ticket[WIDE ? A.phase : 0];
+    const int t0 = WIDE ? A.t0 : 0, t1 = WIDE ? A.t1 : 2 * nn;
+    if (tid == 0) s_tk = t0 + (int)atomicAdd(ticket, 1u);
     __syncthreads();
     for (;;) {
         const int tk = s_tk;
-        if (tk >= A.t1) break;
+        if (tk >= t1) break;
         // the next ticket is taken now and used after this step: the atomic's
         // latency overlaps the step (the block runs both steps in order)
         unsigned next = 0;
-        if (tid == 0) next = A.t0 + atomicAdd(ticket, 1u);
+        if (tid == 0) next = t0 + atomicAdd(ticket, 1u);
         const bool fwd = tk < nn;
         CH_TRACE(tk, 0);
         const int J = fwd ? A.order[tk] : A.order[2 * nn - 1 - tk];
@@ -919,7 +923,7 @@ k_chol_sweep(SweepArgs A) {
         }
         __syncthreads();
     }
-    if (!A.last) return;
+    if (WIDE && !A.last) return;
     // r = bp - C x once every backward step is done; per-block sums of r.r
     CH_TRACE(2 * nn + blockIdx.x, 0);
     if (tid == 0) s_ok = wait_until(&ctl->bcount, (unsigned)nn, true, ctl);
@@ -1485,7 +1489,7 @@ static int chol_sweep_kernels(tp_mesh* m, int nsweep, int rgrid, double* partr, 
             const int grid = std::max(1, std::min(want, most));
             if (want == 0) continue;
             const size_t smem = big ? c->solve_smem[K] : c->small_smem[K];
-            if (c->wide)
+            if (c->wide || parts)
                 k_chol_sweep<K, true><<<grid, CHS_T, smem, st>>>(A);
             else
                 k_chol_sweep<K, false><<<grid, CHS_T, smem, st>>>(A);
