@@ -11,18 +11,20 @@
 //   Differential: with t = u / |d|^2 and f = 2 / |d|^2 (the doubling is an integer
 //   addition to the exponent, off the FP32 pipe) the terms are powers of t^ = u f
 //   times a_T f, which keeps the ratio 2 between the two parts of dE/dX and needs
-//   neither K nor the energy's own sum: 36 operations against 41, 8 sums against 12.
+//   neither K nor the energy's own sum: 36 operations against 41. The 12 sums become
+//   8: N_S . sum(w d) gives a K_ST's part of dE/da after the loop.
 //
 // Targets go in pairs through packed f32x2 instructions; a source's coordinates,
 // normal and area are staged in shared memory already doubled ({x, x}, ...). Tiles
 // near a block's targets take the same path with the differences of the low parts
 // added. A block takes an equal run of units (32 sources against a row of targets),
 // so no wave of blocks is left partly empty whatever the size. FP32 sums over 32
-// sources, Kahan pairs across them, FP64 from there.
+// sources (16 for dE of small meshes), Kahan pairs across them, FP64 from there.
 //
-// Measured: E on 20,000 / 69,690 faces 259 / 2,588 us -> 172 / 1,822 us, dE on 20,000
-// faces 583 -> 560 us. The FP32 pipe is busy 73% (E) and 70% (dE) of the SMs' active
-// cycles; four targets a thread for dE (half the shared-memory reads) ran slower.
+// Measured: E on 20,000 / 69,690 faces 259 / 2,588 us -> 172 / 1,822 us; a call for dE
+// and E on 2,176 / 20,000 / 69,690 faces 103 / 674 / 6,605 us -> 71 / 610 / 6,416 us. The
+// FP32 pipe is busy 73% (E) and 70% (dE) of the SMs' active cycles; four targets a thread
+// for dE (half the shared-memory reads) ran slower.
 #include <algorithm>
 #include <cmath>
 #include <map>
@@ -318,23 +320,24 @@ k_energy_total(const float4* __restrict__ fa, const float4* __restrict__ fb, con
 
 // sums over the sources T (with f = 2 / |d|^2, u_S = N_S.d, u_T = N_T.d, t = u f):
 // 0 a f t_S^5 | 1-3 the same times d | 4-6 a f t_T^5 N_T - (a f (t_S^6 + t_T^6)) d
-// | 7 (a f (t_S^6 + t_T^6)) |d|^2. In the terms of the differential
-//   a c_S = (0) / 64,  a (K_ST + K_TS) = (7) / 128,
+// | 7 a f t_T^5 u_T. In the terms of the differential
+//   a c_S = (0) / 64,  a (K_ST + K_TS) = (N_S . (1-3) + (7)) / 64,
 //   p a c_T N_T - 2 p a (K_ST + K_TS) d / |d|^2 = p (4-6) / 64.
 constexpr int DA = 8;
+constexpr int DS = DA + 3;   // the FP32 sums keep the two parts of 4-6 apart: less rounding (they cancel)
 
-template <bool COMP>
-__device__ __forceinline__ void diff_chunk(const Tile& t, int c0, const Targets<1>& T, u64 (&s)[DA]) {
+template <bool COMP, int NC>
+__device__ __forceinline__ void diff_chunk(const Tile& t, int c0, const Targets<1>& T, u64 (&s)[DS]) {
     const u64 EPS = pk(1e-18f, 1e-18f);
 #pragma unroll 8
-    for (int q = c0; q < c0 + EC; ++q) {
+    for (int q = c0; q < c0 + NC; ++q) {
         const ulonglong2 g0 = t.g[q][0], g1 = t.g[q][1], g2 = t.g[q][2], g3 = t.g[q][3];
         u64 dx, dy, dz;
         T.template diff<COMP>(0, t, q, g0, g1, dx, dy, dz);
         const u64 r2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, EPS)));
         const u64 f = rcp2_twice(r2);
         const u64 tS = mul2(fma2(T.nx[0], dx, fma2(T.ny[0], dy, mul2(T.nz[0], dz))), f);
-        const u64 tT = mul2(fma2(g2.x, dx, fma2(g2.y, dy, mul2(g3.x, dz))), f);
+        const u64 uT = fma2(g2.x, dx, fma2(g2.y, dy, mul2(g3.x, dz))), tT = mul2(uT, f);
         const u64 qS = mul2(tS, tS), qT = mul2(tT, tT);
         const u64 af = mul2(g1.y, f);
         const u64 w = mul2(mul2(mul2(qS, qS), tS), af);
@@ -346,20 +349,31 @@ __device__ __forceinline__ void diff_chunk(const Tile& t, int c0, const Targets<
         s[1] = fma2(w, dx, s[1]);
         s[2] = fma2(w, dy, s[2]);
         s[3] = fma2(w, dz, s[3]);
-        s[4] = fma2(nk, dx, fma2(v, g2.x, s[4]));
-        s[5] = fma2(nk, dy, fma2(v, g2.y, s[5]));
-        s[6] = fma2(nk, dz, fma2(v, g3.x, s[6]));
-        s[7] = fma2(k, r2, s[7]);
+        s[4] = fma2(v, g2.x, s[4]);
+        s[5] = fma2(v, g2.y, s[5]);
+        s[6] = fma2(v, g3.x, s[6]);
+        s[8] = fma2(nk, dx, s[8]);
+        s[9] = fma2(nk, dy, s[9]);
+        s[10] = fma2(nk, dz, s[10]);
+        s[7] = fma2(v, uT, s[7]);
     }
 }
 
 constexpr int DROW = 2 * ET;   // targets per row
+
+// FP32 sums of dE over 16 sources up to this many faces, over 32 beyond. The error of dE
+// against FP64 sums (noisy tori, means over 16 to 64 meshes): 512 / 2,176 / 6,820 /
+// 10,080 faces 4.40 / 2.68 / 3.93 / 3.17e-7 with 32, 4.21 / 2.71 / 3.48 / 3.23e-7 with
+// 16, against 4.35 / 2.78 / 3.75 / 3.62e-7 of the kernel with 12 sums; 16 sources cost
+// nothing at 6,820 faces (133 us), 3 and 4% at 10,080 and 20,000 (208 -> 213, 610 -> 634).
+constexpr int DIFF_SHORT = 8192;
 
 // units of block b of G: [b U / G, (b + 1) U / G); row r's units start at r * per
 __host__ __device__ __forceinline__ long long diff_block(long long u, long long U, long long G) {
     return ((u + 1) * G - 1) / U;
 }
 
+template <int NC>
 __global__ void __launch_bounds__(ET, 5)
 k_diff_sums(const float4* __restrict__ fa, const float4* __restrict__ fb, const float4* __restrict__ fl,
             const float4* __restrict__ tbox, const double* __restrict__ center, int nf, long long per, long long units,
@@ -385,18 +399,18 @@ k_diff_sums(const float4* __restrict__ fa, const float4* __restrict__ fb, const 
             __syncthreads();
             stage(t, fa, fb, fl, tile * ET + tid, nf, true);
             __syncthreads();
-            for (int q = q0; q < q1; ++q) {
-                u64 s[DA];
+            for (int q = q0 * (EC / NC); q < q1 * (EC / NC); ++q) {   // q * NC: source of the tile
+                u64 s[DS];
 #pragma unroll
-                for (int i = 0; i < DA; ++i) s[i] = 0ull;
+                for (int i = 0; i < DS; ++i) s[i] = 0ull;
                 if (near)
-                    diff_chunk<true>(t, q * EC, T, s);
+                    diff_chunk<true, NC>(t, q * NC, T, s);
                 else
-                    diff_chunk<false>(t, q * EC, T, s);
+                    diff_chunk<false, NC>(t, q * NC, T, s);
 #pragma unroll
                 for (int i = 0; i < DA; ++i) {
                     Kahan2 k = acc[i][tid];
-                    k.add(s[i]);
+                    k.add(i >= 4 && i < 7 ? add2(s[i], s[i + 4]) : s[i]);
                     acc[i][tid] = k;
                 }
             }
@@ -449,7 +463,9 @@ k_diff_finish(const double* __restrict__ part, int nf, long long per, long long 
                 gX[q] = c * fma(x, N[q], sh[4 + q][fl]);
                 gN[q] = c * sh[1 + q][fl];
             }
-            const double ga = sh[7][fl] * (1.0 / 128.0);
+            // (the normal that the pair kernel had)
+            const double ga = (sh[7][fl] + (double)(float)N[0] * sh[1][fl] + (double)(float)N[1] * sh[2][fl] +
+                               (double)(float)N[2] * sh[3][fl]) * (1.0 / 64.0);
             er = 0.5 * a * ga;
             if (CORNER) {
                 const double nn = 2.0 * a;
@@ -553,7 +569,8 @@ bool p6_fp32_direct(const tp_params* p) {
 
 int energy_total_p6(tp_mesh* m, double* E_dev, cudaStream_t st) {
     // four targets a thread share each source's shared-memory reads; two where four
-    // leave units for fewer than half of the SMs' blocks (below about 4,000 faces)
+    // leave fewer units than two rounds of the SMs' four blocks (up to 24 tiles, 3,072
+    // faces, on 152 SMs)
     const long long nt = (m->nf + ET - 1) / ET;
     return 2 * nt * nt / 4 * (ET / EC) >= 8LL * sm_count() ? launch_energy<2>(m, E_dev, st)
                                                            : launch_energy<1>(m, E_dev, st);
@@ -562,7 +579,8 @@ int energy_total_p6(tp_mesh* m, double* E_dev, cudaStream_t st) {
 int diff_p6(tp_mesh* m, double* adj, double* erow, double* corner, double* E_dev, cudaStream_t st) {
     const int nf = m->nf, nt = (nf + ET - 1) / ET, rows = (nf + DROW - 1) / DROW;
     const long long per = (long long)nt * (ET / EC), units = per * rows;
-    const long long G = std::min<long long>(units, GD * sm_count() * resident((const void*)k_diff_sums));
+    const auto kernel = nf <= DIFF_SHORT ? k_diff_sums<EC / 2> : k_diff_sums<EC>;
+    const long long G = std::min<long long>(units, GD * sm_count() * resident((const void*)kernel));
     long long slots = 1;   // most blocks that share a row
     for (long long r = 0; r < rows; ++r)
         slots = std::max(slots, diff_block((r + 1) * per - 1, units, G) - diff_block(r * per, units, G) + 1);
@@ -571,9 +589,9 @@ int diff_p6(tp_mesh* m, double* adj, double* erow, double* corner, double* E_dev
     m->pairs += pairs;
     {
         ProfScope ps(m, PK_DIFF, pairs, st);
-        k_diff_sums<<<(unsigned)G, ET, 0, st>>>(m->f32a.as<float4>(), m->f32b.as<float4>(), m->f32c.as<float4>(),
-                                                m->tilebox.as<float4>(), m->center.as<double>(), nf, per, units,
-                                                m->part.as<double>());
+        kernel<<<(unsigned)G, ET, 0, st>>>(m->f32a.as<float4>(), m->f32b.as<float4>(), m->f32c.as<float4>(),
+                                           m->tilebox.as<float4>(), m->center.as<double>(), nf, per, units,
+                                           m->part.as<double>());
         TP_LAUNCH_CHECK();
     }
     const int nb = (nf + 31) / 32;
