@@ -45,15 +45,7 @@ __device__ __forceinline__ float rcp_(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-// FP64 reciprocal: the 20-bit approximation and one third-order step, three
-// FP64 operations in place of the division's sequence (the FP64 pipe issues
-// two lanes a cycle and SM and bounds every FP64 kernel); error below one ulp
-__device__ __forceinline__ double rcp_(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return __double2hiint(x) == 0x7ff00000 ? 0.0 : fma(y, fma(e, e, e), y);
-}
+__device__ __forceinline__ double rcp_(double x) { return __double2hiint(x) == 0x7ff00000 ? 0.0 : rcp64(x); }
 
 __device__ __forceinline__ float lg2_(float x) {
     float r;

@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "fp64_math.cuh"
 #include "tp.h"
 
 // ---------------------------------------------------------------------------
@@ -74,45 +75,6 @@ int sm_count();
 // far away, so that every kernel value at them is finite and zero times it is zero. At
 // the origin, the frame's centre, a face within 4e-7 of it would make |d|^-6 infinite.
 constexpr float PAD_X = 1e18f;
-
-// ---------------------------------------------------------------------------
-// FP64 divisions and roots in few operations
-// ---------------------------------------------------------------------------
-//
-// The FP64 pipe issues two lanes a cycle and SM, and the compiler's division and
-// square root are sequences of 10 to 20 operations on it. These start from the
-// 20-bit approximations and take one third-order step; a quotient or root then gets
-// a residual correction, which makes it the correctly rounded one but for rare ties.
-
-// reciprocal of a normal x
-__device__ __forceinline__ double rcp64(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-// a / b with r = 1 / b (to about an ulp)
-__device__ __forceinline__ double div64(double a, double b, double r) {
-    const double q = a * r;
-    return fma(fma(-q, b, a), r, q);
-}
-// sqrt(x), and its reciprocal in *r; x outside [1e-280, 1e280] takes the functions
-__device__ __forceinline__ double sqrt64(double x, double* r) {
-    if (!(x > 1e-280 && x < 1e280)) {
-        const double s = sqrt(x);
-        *r = 1.0 / s;
-        return s;
-    }
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x * y, y, 1.0);
-    y = fma(y * e, fma(e, 0.375, 0.5), y);
-    const double s0 = x * y;
-    const double s = fma(fma(-s0, s0, x), 0.5 * y, s0);
-    *r = fma(y, fma(-s, y, 1.0), y);
-    return s;
-}
-__device__ __forceinline__ double third64(double x) { return div64(x, 3.0, 1.0 / 3.0); }
 
 // ---------------------------------------------------------------------------
 // bounding box of points in one launch
