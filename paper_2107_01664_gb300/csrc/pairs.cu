@@ -45,74 +45,11 @@ __device__ __forceinline__ float rcp_(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ double rcp_(double x) { return __double2hiint(x) == 0x7ff00000 ? 0.0 : rcp64(x); }
+__device__ __forceinline__ double rcp_(double x) { return rcp64_inf(x); }
 
-__device__ __forceinline__ float lg2_(float x) {
-    float r;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float ex2_(float x) {
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 // x^y for x >= 0 (x = 0 gives 0 for y > 0)
 __device__ __forceinline__ float pow_(float x, float y) { return ex2_(y * lg2_(x)); }
 __device__ __forceinline__ double pow_(double x, double y) { return pow(x, y); }
-
-// x^{-a} in FP64 for a rational a = k / n with a small n (n = 0: pow). With
-// u = x^{-1/n} from the FP32 MUFU (relative error about 1e-6) and e = 1 - x u^n,
-//   x^{-a} = u^k (1 - e)^{-a} = u^k (1 + a e + a (a+1)/2 e^2 + a (a+1) (a+2)/6 e^3 + ..),
-// whose next term is below 1e-18. About 12 FP64 operations at n = 3 (p = 6) in
-// place of about 100 for pow. x outside FP32's range takes pow.
-struct RootPow {
-    int n = 0, k = 0;
-    float inv = 0.f;   // -1 / n
-    double a = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0;
-};
-
-__device__ __forceinline__ double ipow_(double u, int k) {   // u^k, k >= 1
-    double r = 1.0, b = u;
-    bool first = true;
-    for (;;) {
-        if (k & 1) {
-            r = first ? b : r * b;
-            first = false;
-        }
-        k >>= 1;
-        if (!k) break;
-        b *= b;
-    }
-    return r;
-}
-
-// x^{-a}; *ix = 1/x. The conversions between FP32 and FP64 would run on the
-// FP64 pipe: normal numbers are converted by shifting the bits instead (x
-// truncated to FP32, which only moves the seed by 2^-23).
-__device__ __forceinline__ double root_pow(double x, const RootPow& rp, double* ix) {
-    const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
-    // 2^-100 <= x < 2^100
-    if (rp.n == 0 || xh - ((1023u - 100u) << 20) >= (200u << 20)) {
-        *ix = rcp_(x);
-        return pow_(x, -rp.a);
-    }
-    const float xf = __uint_as_float(__funnelshift_l(xl, xh, 3) - ((1023u - 127u) << 23));
-    const unsigned uf = __float_as_uint(ex2_(lg2_(xf) * rp.inv));
-    const double u = __hiloint2double((int)((uf >> 3) + ((1023u - 127u) << 20)), (int)(uf << 29));
-    double un, uk;
-    if (rp.n == 3) {
-        const double u2 = u * u, u4 = u2 * u2;
-        un = u2 * u;
-        uk = rp.k == 5 ? u4 * u : rp.k == 4 ? u4 : ipow_(u, rp.k);
-    } else {
-        un = ipow_(u, rp.n);
-        uk = ipow_(u, rp.k);
-    }
-    const double e = fma(-x, un, 1.0);
-    *ix = fma(un, fma(e, fma(e, e, e), e), un);
-    return fma(uk * e, fma(fma(rp.c3, e, rp.c2), e, rp.c1), uk);
-}
 
 // smallest |d|^2 treated as a real pair; the self pair has d = 0 exactly
 template <typename T> __device__ __forceinline__ T tiny_r2();
@@ -1553,7 +1490,7 @@ k_apply_combine(const double* __restrict__ part, int nsplit, int nf, const d4* _
     double hV[3] = {0.0, 0.0, 0.0}, hU = 0.0;
     const bool mine = has && c < KC && col0 + c < k;
     if (has && c == KC) {   // the areas' sums
-        const double ia = 1.0 / a;
+        const double ia = a > 1e-280 && a < 1e280 ? rcp64(a) : 1.0 / a;
         double hi = 0.0, lo = 0.0;
         // four splits' loads in flight: a small mesh has many splits and few blocks here
         // (A, one column, one call with its synchronisation: 2,400 faces 77 us, 8,140 184)
@@ -1571,8 +1508,8 @@ k_apply_combine(const double* __restrict__ part, int nsplit, int nf, const d4* _
                 lo += y[i];
             }
         }
-        s_hi[fl] = hi * ia;
-        s_lo[fl] = lo * ia;
+        s_hi[fl] = div64(hi, a, ia);
+        s_lo[fl] = div64(lo, a, ia);
     } else if (mine) {
         for (int s0 = 0; s0 < nsplit; s0 += 4) {
             double x[4][4];
@@ -1608,28 +1545,6 @@ k_apply_combine(const double* __restrict__ part, int nsplit, int nf, const d4* _
         if (L::HIGH) g += gr[3 * cr] * zV[0] + gr[3 * cr + 1] * zV[1] + gr[3 * cr + 2] * zV[2];
         corner[((size_t)S * 3 + cr) * k + col0 + c] = a2 * g;
     }
-}
-
-// the FP64 power plan of |d|^{-2s}, s = 2 - 2/p (or, for L, of |d|^{-2(1 + 2/p)}):
-// rational when 2 n / p is a whole number for some n <= 16 (p = 6: n = 3; 4.5: n = 9)
-static RootPow root_plan(double p, bool op_l) {
-    RootPow r;
-    const double q = 2.0 / p;
-    r.a = op_l ? 3.0 - (2.0 - q) : 2.0 - q;
-    for (int n = 1; n <= 16; ++n) {
-        const double m = std::round(q * n);
-        if (std::fabs(q * n - m) > 4e-16 * n) continue;
-        const int k = op_l ? n + (int)m : 2 * n - (int)m;
-        r.n = n;
-        r.k = k;
-        r.a = (double)k / n;
-        r.inv = -1.f / (float)n;
-        break;
-    }
-    r.c1 = r.a;
-    r.c2 = 0.5 * r.a * (r.a + 1.0);
-    r.c3 = r.a * (r.a + 1.0) * (r.a + 2.0) / 6.0;
-    return r;
 }
 
 template <typename T, int OP, int KC>

@@ -1,4 +1,5 @@
-// Test driver of fp64_math.cuh: one function over arrays.
+// Test driver of fp64_math.cuh: one function over arrays (the power's plan from b[0]: p,
+// negative for L).
 //   in  file: int32 op, n; float64 a[n], b[n]
 //   out file: float64 x[n], y[n] (y: the second result, where the function has one)
 #include <cmath>
@@ -7,7 +8,7 @@
 
 #include "fp64_math.cuh"
 
-__global__ void run(int op, int n, const double* a, const double* b, double* x, double* y) {
+__global__ void run(int op, int n, const double* a, const double* b, double* x, double* y, tp::RootPow rp) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double u = 0.0, v = 0.0;
@@ -15,6 +16,8 @@ __global__ void run(int op, int n, const double* a, const double* b, double* x, 
     if (op == 1) u = tp::div64(a[i], b[i], tp::rcp64(b[i])), v = a[i] / b[i];
     if (op == 2) u = tp::sqrt64(a[i], &v);
     if (op == 3) u = tp::third64(a[i]), v = a[i] / 3.0;
+    if (op == 4) u = tp::root_pow(a[i], rp, &v);
+    if (op == 5) u = pow(a[i], -rp.a), v = rp.a;
     x[i] = u;
     y[i] = v;
 }
@@ -32,7 +35,8 @@ int main(int argc, char** argv) {
     if (cudaMalloc(&d, 32 * n) != cudaSuccess ||
         cudaMemcpy(d, h.data(), 16 * n, cudaMemcpyHostToDevice) != cudaSuccess)
         return 3;
-    run<<<(unsigned)((n + 127) / 128), 128>>>(hdr[0], (int)n, d, d + n, d + 2 * n, d + 3 * n);
+    run<<<(unsigned)((n + 127) / 128), 128>>>(hdr[0], (int)n, d, d + n, d + 2 * n, d + 3 * n,
+                                            tp::root_plan(std::fabs(h[n]), h[n] < 0.0));
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemcpy(h.data(), d + 2 * n, 16 * n, cudaMemcpyDeviceToHost) != cudaSuccess)
         return 3;

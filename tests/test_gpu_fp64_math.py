@@ -5,8 +5,13 @@ next to powers of two and to 3/2, and arguments around the range switches.
 Bounds: the reciprocal's series leaves 2^-72, so its last rounding decides: 0.5 ulp and
 a 2^-18 of one. Quotients and roots are the rounded ones but where they lie within
 2^-50 ulp of the middle of two numbers (next to powers of two some do), that is, within
-0.5 ulp and a 2^-50 of one."""
+0.5 ulp and a 2^-50 of one. The power x^-a, a = k / n, against 50 decimal digits: the
+first term left out of the series is 2^-56 relative (0.08 ulp). At n = 3 the rounding of
+one product and the last one remain, at n = 2 these at most, at other n those of up to
+five products with weights of at most one, half an ulp each; its reciprocal 1 / x leaves
+2^-58. Without a plan it is pow, which CUDA documents at 2 ulp."""
 import subprocess
+from decimal import Decimal, localcontext
 from fractions import Fraction
 
 import numpy as np
@@ -110,3 +115,29 @@ def test_third(call):
     y, cuda = call(3, x)
     assert np.array_equal(cuda, x / 3.0)
     assert rounded(y, cuda, lambda i: Fraction(float(x[i])) / 3)
+
+
+@pytest.mark.parametrize("p,kn,kl", [(6.0, (3, 5), (3, 4)), (3.0, (3, 4), (3, 5)), (4.5, (9, 14), (9, 13)),
+                                     (4.0, (2, 3), (2, 3)), (5.0, (5, 8), (5, 7)), (2.5, (5, 6), (5, 9)),
+                                     (32.0 / 13.0, (16, 19), (16, 29)), (3.7, None, None)])
+@pytest.mark.parametrize("low", [False, True])
+@pytest.mark.parametrize("lo,hi", [(-3, 3), (-40, 20), (-100, 100), (-140, -100), (100, 140)])
+def test_rational_power(call, p, kn, kl, low, lo, hi):      # 2^-100 .. 2^100: the plan's range
+    x = np.abs(numbers(6, lo, hi, 1500))
+    b = np.full_like(x, -p if low else p)
+    y, ix = call(4, x, b)
+    n, k = (kl if low else kn) or (0, 0)
+    a = float(call(5, x, b)[1][0])
+    with localcontext() as c:
+        c.prec = 50
+        e = Decimal(k) / Decimal(n) if n else Decimal(a)
+        want = [(-e * Decimal(float(v)).ln()).exp() for v in x]
+        err = np.array([abs(float((Decimal(float(u)) - w) / Decimal(float(np.spacing(u))))) for u, w in zip(y, want)])
+        inv = np.array([abs(float((Decimal(float(u)) - 1 / Decimal(float(v))) / Decimal(float(np.spacing(u)))))
+                        for u, v in zip(ix, x)])
+    # outside its range, and without a plan, pow to the rounded exponent a: a's own rounding
+    # (2^-54 a) adds 2^-54 a |ln x| relative
+    plan = n > 0 and -100 <= lo and hi <= 100
+    bound = (1.08 if n <= 3 else 3.08) if plan else 2.0 + a * np.abs(np.log(x))
+    assert np.all(err <= bound), err.max()
+    assert inv.max() <= 0.53
