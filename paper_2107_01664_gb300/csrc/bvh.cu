@@ -620,12 +620,25 @@ __device__ __forceinline__ float wmax(float x) {
 // their own, in order), and k_bh_list_compact copies them to their places once the
 // counts are summed. A traversal is bound by the latency of its dependent node
 // loads, the copy by memory, so this takes half the time of counting first and
-// writing in a second traversal (327,680 faces: 2.76 -> 1.26 ms). A pool that turns
-// out too small only costs the second traversal. Two warps a block: the groups'
+// writing in a second traversal (327,680 faces: 2.76 -> 1.26 ms). Where the pool
+// turns out too small (rough surfaces) the counts are right all the same, and a
+// second traversal (DIRECT) writes the entries to their places; the pool then grows
+// for the mesh's next tree, never past BHL_POOL_MAX. Two warps a block: the groups'
 // lengths differ by several times and a block holds its place until its last warp
 // is done.
 constexpr int BHL_CHUNK = 64;
 constexpr int BHL_WARPS = 2;
+constexpr size_t BHL_CHUNK_BYTES = sizeof(int2) * (BHL_CHUNK + 1);   // the entries and the chunk's place
+constexpr size_t BHL_POOL_MAX = (size_t)2 << 30;
+
+// chunks of a mesh's first pool: 2,048 entries a group at theta = 0.5 (about 1,150 are
+// used on a smooth surface of 327,680 faces), more at smaller theta (entries go like
+// theta^-2)
+static size_t bhl_first_chunks(int nf, double theta) {
+    const double ngroups = (nf + BHL_GROUP - 1) / BHL_GROUP;
+    const double per_group = 32.0 * std::min(16.0, std::max(1.0, 0.25 / (theta * theta)));
+    return std::min((size_t)(per_group * ngroups + 64.0), BHL_POOL_MAX / BHL_CHUNK_BYTES);
+}
 
 struct BhListCtl {
     unsigned cursor;    // chunks handed out (also past the pool's end)
@@ -633,10 +646,14 @@ struct BhListCtl {
     unsigned long long inter;
 };
 
+// DIRECT = false: counts and the pool's chunks; true: the entries to far_out and
+// near_out at the offsets `off` of the counts that the first traversal left
+template <bool DIRECT>
 __global__ void __launch_bounds__(32 * BHL_WARPS)
 k_bh_list(const BvhNode* __restrict__ node, const FaceBox* __restrict__ fbox, int nf, float theta2, int cap,
           long long* __restrict__ cnt, int2* __restrict__ pool, int2* __restrict__ info, unsigned nchunks,
-          BhListCtl* __restrict__ ctl) {
+          BhListCtl* __restrict__ ctl, const long long* __restrict__ off, int2* __restrict__ far_out,
+          int2* __restrict__ near_out) {
     extern __shared__ int2 lstack[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int ngroups = (nf + BHL_GROUP - 1) / BHL_GROUP;
@@ -669,6 +686,13 @@ k_bh_list(const BvhNode* __restrict__ node, const FaceBox* __restrict__ fbox, in
     unsigned chunk[2] = {0u, 0u};
     auto append = [&](int kind, unsigned who, int2 e) {   // lanes in `who` each append e, in lane order
         const int k = __popc(who);
+        if constexpr (DIRECT) {
+            const size_t row = (size_t)kind * (ngroups + 1) + g;
+            const long long at = off[row] + n[kind] + __popc(who & lt);
+            if (((who >> lane) & 1u) && at < off[row + 1]) (kind ? near_out : far_out)[at] = e;
+            n[kind] += k;
+            return;
+        }
         const int p0 = n[kind], c0 = p0 / BHL_CHUNK, c1 = (p0 + k - 1) / BHL_CHUNK;
         const bool start = p0 % BHL_CHUNK == 0, cross = c1 != c0;
         unsigned nxt = 0u;
@@ -776,6 +800,7 @@ k_bh_list(const BvhNode* __restrict__ node, const FaceBox* __restrict__ fbox, in
         }
         __syncwarp();
     }
+    if (DIRECT) return;
     for (int o = 16; o > 0; o >>= 1) ninter += __shfl_xor_sync(0xffffffffu, ninter, o);
     if (lane == 0) {
         if (over) atomicExch(&ctl->err, 1);
@@ -843,42 +868,31 @@ int bh_lists(tp_mesh* m, const tp_params* p, cudaStream_t st, BhLists* out, bool
     BhListCtl* ctl = reinterpret_cast<BhListCtl*>(counts + 2 * (ngroups + 1));
     void* scan_ws = reinterpret_cast<char*>(m->bhl_cnt.ptr) + sizeof(long long) * head;
     const float theta2 = (float)(p->theta * p->theta);
-    // chunks of the pool: 2,048 entries a group at theta = 0.5 (about 1,150 are used
-    // on a smooth surface of 327,680 faces), more at smaller theta
-    // (entries go like theta^-2), 2 GB at most; a second round knows the number
-    const double per_group = 32.0 * std::min(16.0, std::max(1.0, 0.25 / (p->theta * p->theta)));
-    constexpr double chunk_bytes = sizeof(int2) * (BHL_CHUNK + 1);
-    double want = std::min(per_group * ngroups + 64.0, 2.0e9 / chunk_bytes);
+    const size_t want = std::max(bhl_first_chunks(nf, p->theta), m->bhl_want);
+    const size_t have = m->bhl_pool.bytes / BHL_CHUNK_BYTES;   // a grown pool is used whole
+    unsigned nchunks = (unsigned)std::max(want, have);
+    if (want > have && ensure(m->bhl_pool, BHL_CHUNK_BYTES * want) != TP_OK) {
+        set_error("");
+        nchunks = 0;                                 // no room for the pool: two traversals
+    }
+    int2* pool = m->bhl_pool.as<int2>();
+    int2* info = pool + (size_t)nchunks * BHL_CHUNK;
+    const int blocks = (ngroups + BHL_WARPS - 1) / BHL_WARPS;
+    TP_CUDA(cudaMemsetAsync(off, 0, sizeof(long long) * head, st));
+    k_bh_list<false><<<blocks, 32 * BHL_WARPS, smem, st>>>(na.node, fbox, nf, theta2, cap, counts, pool, info, nchunks,
+                                                           ctl, nullptr, nullptr, nullptr);
+    TP_LAUNCH_CHECK();
+    // counts -> exclusive offsets (the extra last entry becomes the total)
+    TP_CUDA(cub::DeviceScan::ExclusiveSum(scan_ws, scan_bytes, counts, off, ngroups + 1, st));
+    TP_CUDA(cub::DeviceScan::ExclusiveSum(scan_ws, scan_bytes, counts + ngroups + 1, off + ngroups + 1, ngroups + 1,
+                                          st));
     BhListCtl h{};
     long long tot[2] = {0, 0};
-    unsigned nchunks = 0;
-    int2 *pool = nullptr, *info = nullptr;
-    for (int round = 0; round < 2; ++round) {
-        const size_t have = (size_t)(m->bhl_pool.bytes / chunk_bytes);   // a grown pool is used whole
-        nchunks = (unsigned)std::min(4.0e9, std::max(want, (double)have));
-        if ((size_t)nchunks > have && ensure(m->bhl_pool, (size_t)(chunk_bytes * nchunks)) != TP_OK) {
-            set_error("");
-            return TP_OK;                            // no room for the pool: the walks serve
-        }
-        pool = m->bhl_pool.as<int2>();
-        info = pool + (size_t)nchunks * BHL_CHUNK;
-        TP_CUDA(cudaMemsetAsync(off, 0, sizeof(long long) * head, st));
-        k_bh_list<<<(ngroups + BHL_WARPS - 1) / BHL_WARPS, 32 * BHL_WARPS, smem, st>>>(
-            na.node, fbox, nf, theta2, cap, counts, pool, info, nchunks, ctl);
-        TP_LAUNCH_CHECK();
-        // counts -> exclusive offsets (the extra last entry becomes the total)
-        TP_CUDA(cub::DeviceScan::ExclusiveSum(scan_ws, scan_bytes, counts, off, ngroups + 1, st));
-        TP_CUDA(cub::DeviceScan::ExclusiveSum(scan_ws, scan_bytes, counts + ngroups + 1, off + ngroups + 1,
-                                              ngroups + 1, st));
-        TP_CUDA(cudaMemcpyAsync(&tot[0], off + ngroups, sizeof(long long), cudaMemcpyDeviceToHost, st));
-        TP_CUDA(cudaMemcpyAsync(&tot[1], off + 2 * ngroups + 1, sizeof(long long), cudaMemcpyDeviceToHost, st));
-        TP_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(h), cudaMemcpyDeviceToHost, st));
-        TP_CUDA(cudaStreamSynchronize(st));
-        if (h.err != 0) return TP_OK;                // a stack overflowed: the walks serve this tree
-        if (h.cursor <= nchunks) break;
-        if (round == 1) return TP_OK;
-        want = h.cursor;
-    }
+    TP_CUDA(cudaMemcpyAsync(&tot[0], off + ngroups, sizeof(long long), cudaMemcpyDeviceToHost, st));
+    TP_CUDA(cudaMemcpyAsync(&tot[1], off + 2 * ngroups + 1, sizeof(long long), cudaMemcpyDeviceToHost, st));
+    TP_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(h), cudaMemcpyDeviceToHost, st));
+    TP_CUDA(cudaStreamSynchronize(st));
+    if (h.err != 0) return TP_OK;                    // a stack overflowed: the walks serve this tree
     // entries are addressed with int offsets inside the kernels' loops
     if (tot[0] >= (1LL << 31) || tot[1] >= (1LL << 31)) return TP_OK;
     if (ensure(m->bhl_far, sizeof(int2) * ((size_t)tot[0] + 1)) != TP_OK ||
@@ -886,7 +900,13 @@ int bh_lists(tp_mesh* m, const tp_params* p, cudaStream_t st, BhLists* out, bool
         set_error("");
         return TP_OK;                                // no room for the lists: the walks serve
     }
-    if (h.cursor) {
+    if (h.cursor > nchunks) {
+        k_bh_list<true><<<blocks, 32 * BHL_WARPS, smem, st>>>(na.node, fbox, nf, theta2, cap, nullptr, nullptr, nullptr,
+                                                              0u, nullptr, off, m->bhl_far.as<int2>(),
+                                                              m->bhl_near.as<int2>());
+        TP_LAUNCH_CHECK();
+        if (nchunks && h.cursor <= BHL_POOL_MAX / BHL_CHUNK_BYTES) m->bhl_want = h.cursor;
+    } else if (h.cursor) {
         k_bh_list_compact<<<(h.cursor + 3) / 4, 128, 0, st>>>(pool, info, h.cursor, ngroups, counts, off,
                                                               m->bhl_far.as<int2>(), m->bhl_near.as<int2>());
         TP_LAUNCH_CHECK();

@@ -348,6 +348,7 @@ struct tp_mesh {
     long long bhl_nfar = 0, bhl_nnear = 0;
     unsigned long long bhl_inter = 0;     // interactions of one evaluation over the lists
     bool bhl_failed = false;              // the lists could not be built for this tree (walk kernels serve)
+    size_t bhl_want = 0;                  // chunks of the pool that the mesh's longest lists so far asked for
     tp::Buf bhl_cnt, bhl_far, bhl_near, bhl_pool;
     // workspaces
     tp::Buf part, part2, scal, corner, wv64, wv32, tmpv[8];

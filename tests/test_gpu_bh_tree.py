@@ -43,3 +43,30 @@ def test_lists_of_different_length_on_one_mesh(lib):
     E = O.energy(V, F)
     assert e[1] == e[3]
     assert abs(e[1] / E - 1) <= TOL
+
+
+@pytest.mark.parametrize("noise,theta,leaf", [(0.3, 0.5, 1), (0.3, 0.25, 1), (0.1, 0.5, 4)])
+def test_lists_longer_than_the_first_pool(lib, noise, theta, leaf):
+    # a crumpled surface, whose lists are several times those of a smooth one: the first
+    # tree's entries are written by a second traversal and the pool is not grown for
+    # them, the next tree finds a pool of the size they asked for. The lists are the same,
+    # so E and the apply are equal bit by bit; the walks (rows of given targets) sum the
+    # same terms in another order
+    from synth import gaussian_noise, torus
+    V, F = torus(200, 50, 1.0, 0.3)
+    V = gaussian_noise(V, noise, 1)
+    u = vertex_vectors(len(V), 3, 8)
+    p = lib.params(theta=theta, leaf_size=leaf)
+    with lib.Context(0) as ctx:
+        with lib.Mesh(V, F, ctx=ctx) as m:
+            E, y, used = [], [], []
+            for _ in range(3):
+                E.append(lib.tp_energy(m, p))
+                y.append(lib.fractional_apply(m, "A", u, p))
+                used.append(ctx.memory()[0])
+                m.set_positions(V)
+            rows = lib.tp_energy_rows(m, np.arange(len(F), dtype=np.int32), p)
+    assert used[0] < used[1] == used[2]
+    assert E[0] == E[1] == E[2]
+    assert np.array_equal(y[0], y[1]) and np.array_equal(y[0], y[2])
+    assert abs(E[0] / rows.sum() - 1) <= TOL
