@@ -827,6 +827,19 @@ k_bh_list_compact(const int2* __restrict__ pool, const int2* __restrict__ info, 
     for (int q = lane; q < len; q += 32) dst[q] = src[q];
 }
 
+// Device bytes of the tree and of what hangs on it: sorted faces and sort keys, nodes,
+// the lists' pool and the lists (as long as the first pool; a surface that is rougher
+// than that holds more), the node sums of an apply on nine columns of A
+size_t bh_footprint_bytes(int nf, int leaf, double theta) {
+    const size_t F = (size_t)nf, nn = 2 * ((F + leaf - 1) / leaf), groups = F / BHL_GROUP + 1;
+    const size_t chunks = bhl_first_chunks(nf, theta);
+    const size_t tree = F * (sizeof(int) + sizeof(FaceBox) + 3 * sizeof(float4)) + F * 8 + 65536 +
+                        std::max(F * 16 + 49200, nn * (sizeof(d4) + 12)) + node_bytes((int)nn) +
+                        nn * (sizeof(NodeShape) + 8);
+    const size_t lists = chunks * (BHL_CHUNK_BYTES + sizeof(int2) * BHL_CHUNK) + groups * 32 + 65536;
+    return tree + lists + 16 * (10 * F + 12 * nn) + 44 * nn + F * 16;
+}
+
 int bh_lists(tp_mesh* m, const tp_params* p, cudaStream_t st, BhLists* out, bool* ok) {
     *ok = false;
     TP_TRY(bvh_build(m, p, st));

@@ -289,24 +289,36 @@ int tp_mesh_destroy(tp_mesh* m) {
 
 size_t tp_mesh_footprint_bytes(int nv, int nf, const tp_params* p) {
     if (nv < 0 || nf < 0) return 0;
-    const int restart = p ? std::max(1, std::min(60, p->gmres_restart)) : 30;
-    size_t F = (size_t)nf, V = (size_t)nv;
-    size_t geom = F * (12 + 4 + 16 + 16 + 32 + 32 + 72) + V * (24 + 4);
-    // cotan CSR (pattern, values, FP32 copy), the preconditioner's within-face
-    // term on the same pattern, and the connected-component tables
-    size_t lap = (7 * V + F) * (4 + 8 + 8) + V * 16 + (7 * V) * 8 + V * 12;
-    size_t bvh = F * (4 + 8 + 16 + 16 + 16) + F * 64;
-    size_t nsplit = 16;
-    size_t pairs = nsplit * F * 14 * 8 + F * (96 + 72 + 72 + 56 + 8);
-    size_t krylov = (size_t)(2 * restart + 1) * 3 * V * 8;
-    size_t vecs = 24 * 3 * V * 8;
+    tp_params d;
+    if (!p) {
+        tp_params_default(&d);
+        p = &d;
+    }
+    const int restart = std::max(1, std::min(60, p->gmres_restart));
+    const size_t F = (size_t)nf, V = (size_t)nv;
+    // faces, positions, vertex -> corner table, face tables, tile boxes
+    const size_t geom = F * (12 + 12 + 16 * 3 + 32 * 2 + 72 + 1) + V * (24 + 4);
+    // cotan CSR (V + 3 F entries: column, value, its FP32 copy, corners, the
+    // preconditioner's within-face values), corner cotangents, component tables
+    const size_t lap = (V + 3 * F) * (4 + 8 + 4 + 8 + 8) + V * (4 + 4 + 8 + 4 + 8 + 12) + F * 48;
+    // per face: FP64 and FP32 source vectors of nine columns, their corner values, the
+    // adjoints and energy rows; then the partial sums of the pair kernels
+    const size_t faces = F * (288 + (p->precision == TP_PREC_FP64 ? 320 : 160) + 216 + 56 + 8);
+    const bool bh = p->theta > 0.0;
+    const size_t sums = bh ? F * 38 * 8 + bh_footprint_bytes(nf, std::max(1, p->leaf_size), p->theta)
+                           : pair_partial_bytes(nf, p) + (p->tensor_cores ? F * 432 + 16384 : 0);
+    // Krylov spaces of three systems (gradient, area, volume) and their packed vectors,
+    // the step's and the preconditioner's vectors, those of CG, results
+    const size_t krylov = ((size_t)(2 * restart + 2) * 3 + 9) * 24 * V;
+    const size_t vecs = (8 * 24 + 2 * 72 + 2 * 72) * V + (p->poisson_solver == TP_POISSON_CHOLESKY ? 0 : 6 * 72 * V);
     // sparse Cholesky (nested dissection on a surface: factor and update
     // matrices grow like V log V; about 190 floats per vertex at 10^4
     // vertices) plus its FP32 and FP64 solve vectors
     size_t chol = 0;
-    if (!p || p->poisson_solver == TP_POISSON_CHOLESKY)
+    if (p->poisson_solver == TP_POISSON_CHOLESKY)
         chol = (size_t)(V * 4.0 * 24.0 * std::log2((double)V + 2.0)) + V * 9 * (4 * 3 + 8 * 3) + V * 64;
-    return geom + lap + bvh + pairs + krylov + vecs + chol;
+    const size_t fixed = (size_t)2 << 20;   // reductions, control blocks, rounding to 256 bytes
+    return geom + lap + faces + sums + krylov + vecs + chol + fixed;
 }
 
 int tp_energy(tp_mesh* m, const tp_params* p, double* E_out, void* stream) {

@@ -576,6 +576,11 @@ int energy_total_p6(tp_mesh* m, double* E_dev, cudaStream_t st) {
                                                            : launch_energy<1>(m, E_dev, st);
 }
 
+long long diff_p6_slots_max(int nf, int sms) {
+    const long long per = (nf + ET - 1) / ET * (long long)(ET / EC), rows = (nf + DROW - 1) / DROW;
+    return std::min(per, GD * sms * 8 / std::max(1LL, rows) + 2);
+}
+
 int diff_p6(tp_mesh* m, double* adj, double* erow, double* corner, double* E_dev, cudaStream_t st) {
     const int nf = m->nf, nt = (nf + ET - 1) / ET, rows = (nf + DROW - 1) / DROW;
     const long long per = (long long)nt * (ET / EC), units = per * rows;

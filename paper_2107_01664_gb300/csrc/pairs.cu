@@ -253,12 +253,11 @@ static int resident_per_sm(const void* fn, int threads, size_t dyn_smem = 0) {
 // the kernel time goes like waves x tiles_per_split. The split count
 // minimises that, plus a small charge per split for the partial sums the
 // FP64 combine reads (a split's partials cost about a twentieth of a tile).
-static Grid make_grid(int nt, int nf, int tt, int per_sm) {
+static Grid make_grid(int nt, int nf, int tt, long slots) {
     Grid g;
     g.bx = (nt + NT * tt - 1) / (NT * tt);
     if (g.bx < 1) g.bx = 1;
     const int ntiles = (nf + NT - 1) / NT;
-    const long slots = (long)std::max(1, per_sm) * sm_count();
     double best = 1e300;
     g.tiles_per_split = ntiles;
     g.nsplit = 1;
@@ -275,6 +274,8 @@ static Grid make_grid(int nt, int nf, int tt, int per_sm) {
     }
     return g;
 }
+
+static long grid_slots(int per_sm) { return (long)std::max(1, per_sm) * sm_count(); }
 
 // FP64 kernels run at the rate of an SM's FP64 pipe however many blocks it
 // holds, so what counts is that every SM gets the same number of tiles. Hence at
@@ -472,7 +473,7 @@ static int launch_energy(tp_mesh* m, const tp_params* p, const int32_t* tl, int 
                          cudaStream_t st) {
     using V4 = typename V4T<T>::type;
     constexpr int TT = sizeof(T) == 4 ? 4 : 2;
-    Grid g = make_grid(nt, m->nf, TT, resident_per_sm((const void*)k_energy<T, true, TT>, NT));
+    Grid g = make_grid(nt, m->nf, TT, grid_slots(resident_per_sm((const void*)k_energy<T, true, TT>, NT)));
     if (sizeof(T) == 8) g = fp64_grid(g, m->nf);
     TP_TRY(ensure(m->part, sizeof(double) * (size_t)g.nsplit * nt));
     const V4* fa = (const V4*)(sizeof(T) == 4 ? m->f32a.ptr : m->f64a.ptr);
@@ -676,7 +677,7 @@ template <typename T>
 static int launch_diff(tp_mesh* m, const tp_params* p, double* adj, double* erow, cudaStream_t st) {
     using V4 = typename V4T<T>::type;
     constexpr int TT = sizeof(T) == 4 ? 2 : 1;
-    Grid g = make_grid(m->nf, m->nf, TT, resident_per_sm((const void*)k_diff<T, false, TT>, NT));
+    Grid g = make_grid(m->nf, m->nf, TT, grid_slots(resident_per_sm((const void*)k_diff<T, false, TT>, NT)));
     if (sizeof(T) == 8) g = fp64_grid(g, m->nf);
     TP_TRY(ensure(m->part, sizeof(double) * (size_t)g.nsplit * NADJ * m->nf));
     const V4* fa = (const V4*)(sizeof(T) == 4 ? m->f32a.ptr : m->f64a.ptr);
@@ -1556,7 +1557,7 @@ static int launch_apply_op(tp_mesh* m, const tp_params* p, const double* v, int 
     const double s = 2.0 - 2.0 / p->p;       // Sobolev order, §2.3
     const double l_exp = 3.0 - s;            // |d|^{-(2 sigma + 2)} = r2^{-(sigma+1)}, sigma = 2 - s
     constexpr int TT = (sizeof(T) == 4 && KC == 3) ? 2 : 1;
-    Grid g = make_grid(nf, nf, TT, resident_per_sm((const void*)k_apply<T, OP, TT, KC>, NT));
+    Grid g = make_grid(nf, nf, TT, grid_slots(resident_per_sm((const void*)k_apply<T, OP, TT, KC>, NT)));
     if (sizeof(T) == 8) g = fp64_grid(g, nf);
     TP_TRY(ensure(m->part, sizeof(double) * (size_t)g.nsplit * L::NA * nf));
     TP_TRY(ensure(m->wv64, sizeof(double) * 4 * KC * (size_t)nf));
@@ -2006,6 +2007,26 @@ k_apply_tc(const float4* __restrict__ fa, const float4* __restrict__ fb, const f
     if (warp == TC_CW) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(TC_TMEM_COLS));
 }
 
+// source splits of k_apply_tc: blocks = target blocks x splits run in waves of `slots`; the
+// time goes like waves x (tiles per split + the fixed cost of a block, about 6 tiles)
+static Grid tc_grid(int nf, long long slots) {
+    const int ntile = (nf + TC_KT - 1) / TC_KT;
+    Grid g;
+    g.bx = (nf + 127) / 128;
+    long long best = -1;
+    for (int ns = 1; ns <= 64 && ns <= ntile; ++ns) {
+        const long long tps = (ntile + ns - 1) / ns;
+        const long long waves = ((long long)g.bx * ns + slots - 1) / slots;
+        const long long cost = waves * (tps + 6);
+        if (best < 0 || cost < best) {
+            best = cost;
+            g.nsplit = ns;
+            g.tiles_per_split = (int)tps;
+        }
+    }
+    return g;
+}
+
 // the A apply on 9 columns with tensor-core accumulation (see k_apply_tc)
 static int launch_apply_tc(tp_mesh* m, const tp_params* p, const double* v, int k, double* y, cudaStream_t st) {
     using L = OpLayout<TP_OP_A, 9>;
@@ -2021,25 +2042,8 @@ static int launch_apply_tc(tp_mesh* m, const tp_params* p, const double* v, int 
     }
     const int per_sm = resident_per_sm((const void*)k_apply_tc, TC_T, TC_SMEM);
     if (per_sm < 1) return fail(TP_ERR_CUDA, "k_apply_tc: shared memory per block not available");
-    // source splits: blocks = target blocks x splits run in waves of per_sm x SMs; the time goes
-    // like waves x (tiles per split + the fixed cost of a block, about 6 tiles)
     const int ntile = (nf + TC_KT - 1) / TC_KT;
-    Grid g;
-    g.bx = (nf + 127) / 128;
-    {
-        const long long slots = (long long)per_sm * sm_count();
-        long long best = -1;
-        for (int ns = 1; ns <= 64 && ns <= ntile; ++ns) {
-            const long long tps_ = (ntile + ns - 1) / ns;
-            const long long waves = ((long long)g.bx * ns + slots - 1) / slots;
-            const long long cost = waves * (tps_ + 6);
-            if (best < 0 || cost < best) {
-                best = cost;
-                g.nsplit = ns;
-                g.tiles_per_split = (int)tps_;
-            }
-        }
-    }
+    const Grid g = tc_grid(nf, grid_slots(per_sm));
     const int tps = g.tiles_per_split;
     TP_TRY(ensure(m->part, sizeof(float2) * (size_t)g.nsplit * L::NA * nf + sizeof(double) * L::NA * (size_t)nf));
     TP_TRY(ensure(m->wv64, sizeof(double) * 4 * 9 * (size_t)nf));
@@ -2108,7 +2112,7 @@ static int launch_apply_wide(tp_mesh* m, const tp_params* p, const double* v, in
     const size_t smem = wide_smem_bytes<OP>();
     const int per_sm = resident_per_sm((const void*)k_apply_wide<OP, CHW>, NT, smem);
     if (per_sm < 1) return fail(TP_ERR_CUDA, "k_apply_wide: shared memory per block not available");
-    Grid g = make_grid(nf, nf, WT, per_sm);
+    Grid g = make_grid(nf, nf, WT, grid_slots(per_sm));
     TP_TRY(ensure(m->part, sizeof(float2) * (size_t)g.nsplit * L::NA * nf + sizeof(double) * L::NA * (size_t)nf));
     TP_TRY(ensure(m->wv64, sizeof(double) * 4 * 9 * (size_t)nf));
     TP_TRY(ensure(m->wv32, sizeof(float4) * L::NW4 * (size_t)nf));
@@ -2661,6 +2665,30 @@ int apply_bh(tp_mesh* m, const tp_params* p, int op, const double* v, int k, dou
                                   : launch_bh_apply_op<TP_OP_L, 3>(m, p, v, k, y, st);
     }
     return fail(TP_ERR_INVALID_ARG, "unknown operator");
+}
+
+// Bytes of the partial sums (m->part) of the direct pair kernels on a mesh of nf faces,
+// at most: the split counts of the differential and of the widest applies for up to
+// eight resident blocks per SM of a GB300 (152 SMs)
+size_t pair_partial_bytes(int nf, const tp_params* p) {
+    constexpr long SMS = 152;
+    const long long nt = (nf + NT - 1) / NT, na = OpLayout<TP_OP_A, 9>::NA, na3 = OpLayout<TP_OP_A, 3>::NA;
+    long long bytes = 0;
+    for (long per_sm = 1; per_sm <= 8; ++per_sm) {
+        if (p->precision == TP_PREC_FP64) {
+            const Grid one = make_grid(nf, nf, 1, per_sm * SMS);
+            const long long even = std::min<long long>(nt, 2 * ((8 * SMS + one.bx - 1) / one.bx));   // fp64_grid
+            bytes = std::max(bytes, std::max<long long>(one.nsplit, even) * na * 8);
+        } else {
+            const long long wide = make_grid(nf, nf, WT, per_sm * SMS).nsplit, one = make_grid(nf, nf, 1, per_sm * SMS).nsplit;
+            bytes = std::max({bytes, (wide + 1) * na * 8, one * na3 * 8});
+        }
+    }
+    // (one block per SM)
+    if (p->precision == TP_PREC_FP32 && p->tensor_cores)
+        bytes = std::max(bytes, (long long)(tc_grid(nf, SMS).nsplit + 1) * na * 8);
+    if (p->precision == TP_PREC_FP32 && p->p == 6.0) bytes = std::max(bytes, diff_p6_slots_max(nf, SMS) * 8 * 8);
+    return (size_t)(bytes * nf);
 }
 
 int apply_op(tp_mesh* m, const tp_params* p, int op, const double* v, int k, double* y, cudaStream_t st) {

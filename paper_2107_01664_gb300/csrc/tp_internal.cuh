@@ -428,12 +428,15 @@ int apply_tc_error(tp_mesh* m, int* gave_up, cudaStream_t st);
 int apply_op(tp_mesh* m, const tp_params* p, int op, const double* v_dev, int k, double* y_dev,
              cudaStream_t st);
 
+size_t pair_partial_bytes(int nf, const tp_params* p);   // of m->part in the direct kernels, at most
+
 // -------- energy.cu --------------------------------------------------------
 // direct sums in FP32 at p = 6 (the default mode): whether p asks for them
 bool p6_fp32_direct(const tp_params* p);
 int energy_total_p6(tp_mesh* m, double* E_dev, cudaStream_t st);   // E of Eq. 10 into a device scalar
 // the face corners' gradients [nf*9] and E (device), or with corner = nullptr the
 // face adjoints [nf*7] and energy rows
+long long diff_p6_slots_max(int nf, int sms);   // partial sums of a face in diff_p6, at most
 int diff_p6(tp_mesh* m, double* adj, double* erow, double* corner, double* E_dev, cudaStream_t st);
 
 // -------- bvh.cu -----------------------------------------------------------
@@ -450,6 +453,7 @@ int bh_counts_read(tp_mesh* m, unsigned long long out[BH_NCOUNT], bool reset, cu
 int bvh_view(tp_mesh* m, const tp_params* p, cudaStream_t st, BvhView* out);   // builds the tree if needed
 // interaction lists of the tree for p->theta (built on first use per tree and
 // theta); *ok = false when they cannot be built (the walk kernels then serve)
+size_t bh_footprint_bytes(int nf, int leaf, double theta);   // tree, lists and their pool, workspaces
 int bh_lists(tp_mesh* m, const tp_params* p, cudaStream_t st, BhLists* out, bool* ok);
 
 // -------- cg.cu ------------------------------------------------------------
