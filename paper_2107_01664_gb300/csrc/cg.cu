@@ -699,12 +699,12 @@ int cg_trace(tp_mesh* m, unsigned long long out[10]) {
 }
 
 int cg_solve(tp_mesh* m, const tp_params* p, const double* b, int k, double* z_out, cudaStream_t st,
-             int* iters, bool deferred) {
+             int* iters, PoissonMode mode) {
     if (k < 1 || k > KMAX) return fail(TP_ERR_INVALID_ARG, "cg: k must be in 1..9");
     TP_TRY(laplacian_values(m, st));
     if (p->poisson_solver == TP_POISSON_CHOLESKY) {
         bool used = false;
-        TP_TRY(chol_solve(m, p, b, k, z_out, st, iters, &used, deferred));
+        TP_TRY(chol_solve(m, p, b, k, z_out, st, iters, &used, mode));
         if (used) return TP_OK;
     }
     // FP64 vectors in both precision modes: with FP32 vectors the Jacobi-CG

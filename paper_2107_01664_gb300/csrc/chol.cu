@@ -1141,10 +1141,12 @@ k_comp_mean(const int* __restrict__ comp_ptr, const int* __restrict__ comp_verts
     if (threadIdx.x == 0) {
         *ticket = 0u;
         if (dflags) {
-            // after the sweeps of a deferred solve: its wait error, and whether
-            // it stopped short of the tolerance
+            // after the sweeps of a deferred solve: its wait error, and whether it stopped
+            // short of the tolerance with more than a hundredth of a right-hand side left
             if (ctl->err) dflags[0] = 1;
-            if (!ctl->done || ctl->stalled) dflags[1] = 1;
+            if (!ctl->done || ctl->stalled)
+                for (int j = 0; j < k; ++j)
+                    if (!(ctl->rr[j] <= 1e-4 * ctl->bb[j])) dflags[1] = 1;
         }
     }
 }
@@ -1183,8 +1185,8 @@ void chol_invalidate(tp_mesh* m) {
     }
 }
 
-int chol_deferred_flags(tp_mesh* m, cudaStream_t st, int* err, int* unconverged, bool reset) {
-    *err = *unconverged = 0;
+int chol_deferred_flags(tp_mesh* m, cudaStream_t st, int* err, int* poor, bool reset) {
+    *err = *poor = 0;
     CholState* c = m->chol;
     if (!c || !c->dflags.ptr) return TP_OK;
     if (!reset) {
@@ -1192,7 +1194,7 @@ int chol_deferred_flags(tp_mesh* m, cudaStream_t st, int* err, int* unconverged,
         TP_CUDA(cudaMemcpyAsync(h, c->dflags.ptr, sizeof(h), cudaMemcpyDeviceToHost, st));
         TP_CUDA(cudaStreamSynchronize(st));
         *err = h[0];
-        *unconverged = h[1];
+        *poor = h[1];
     }
     TP_CUDA(cudaMemsetAsync(c->dflags.ptr, 0, 2 * sizeof(int), st));
     return TP_OK;
@@ -1542,8 +1544,9 @@ static int sweep_graph(tp_mesh* m, int rgrid, double* partr, double tol2, int ca
 
 template <int K>
 static int chol_run(tp_mesh* m, const tp_params* p, const double* b, double* z_out, cudaStream_t st, int* iters,
-                    bool* handed_off, bool deferred) {
+                    bool* handed_off, PoissonMode mode) {
     CholState* c = m->chol;
+    const bool deferred = mode == POISSON_DEFERRED;
     if (deferred && !c->pivot_known) {
         // the factor's pivot check, once per factorisation
         int bp = 0;
@@ -1587,18 +1590,23 @@ static int chol_run(tp_mesh* m, const tp_params* p, const double* b, double* z_o
     CholState::SweepGraph* g = nullptr;
     TP_TRY(sweep_graph<K>(m, rgrid, partr, tol2, cap, &g));
     if (deferred) {
-        // no host read: the sweeps that cg_tol needs, then the flags; the
-        // caller reads them once per step. Measured digits of |r|/|b| (9
-        // columns): at least four after the first sweep (torus_20k,
-        // linked_tori_50k, icosphere_l3), about three more per sweep after it.
+        // no host read: a fixed number of sweeps for cg_tol, then the flags, which
+        // the caller reads. Measured digits of |r|/|b| (9 columns, random b): at
+        // least four after the first sweep on up to 25,000 vertices (torus_20k,
+        // linked_tori_50k, icosphere_l3), 2.5 to 3.5 on 40,000 to 120,000 (tori, linked
+        // tori), and two to three more per sweep after it.
         if (!c->dflags.ptr) {
             TP_TRY(ensure(c->dflags, 4 * sizeof(int)));
             TP_CUDA(cudaMemsetAsync(c->dflags.ptr, 0, 4 * sizeof(int), st));   // fresh memory holds garbage
         }
-        // Larger meshes: 2.5 and 1.5 (163,842 vertices: 1e-4 in two sweeps, 1e-9 in
-        // four; 655,362: 1e-4 in three, 1e-6 in four).
+        // Larger meshes: 2.5 and 1.5. 130,200 to 182,000 vertices, smooth or with noise up
+        // to 0.4 edges: 1e-4 in two sweeps (once three: a torus of 1,400 x 110, nine columns),
+        // 1e-6 in three (once four), 1e-9 in four to six; 655,362: 1e-4 in three, 1e-6 in four.
+        // The line lies where the former limit of the factor was: below it the flexible method
+        // has always gone on with what the fewer sweeps give.
         const double digits = -std::log10(std::max(p->cg_tol, 1e-300));
-        const double first = nv <= 120000 ? 4.0 : 2.5, next = nv <= 120000 ? 3.0 : 1.5;
+        const bool large = nv > CHOL_LARGE_NV;
+        const double first = large ? 2.5 : 4.0, next = large ? 1.5 : 3.0;
         const int sweeps = std::min(cap, 1 + std::max(0, (int)std::ceil((digits - first) / next)));
         const int graphs = sweeps / CH_SWEEPS_PER_GRAPH;
         for (int gi = 0; gi < graphs; ++gi) {
@@ -1632,7 +1640,12 @@ static int chol_run(tp_mesh* m, const tp_params* p, const double* b, double* z_o
     }
     if (iters) *iters = h.iters;
     if (h.err) return fail(TP_ERR_TIMEOUT, "cotan solve: a wait of the factorised sweep gave up");
-    if (h.bad_pivot || h.stalled || !h.done) {
+    bool good = h.done && !h.stalled;
+    if (mode == POISSON_LOOSE && !good) {
+        good = true;
+        for (int j = 0; j < K; ++j) good = good && h.rr[j] <= 1e-4 * h.bb[j];
+    }
+    if (h.bad_pivot || !good) {
         *handed_off = true;
         return TP_OK;
     }
@@ -1643,7 +1656,7 @@ static int chol_run(tp_mesh* m, const tp_params* p, const double* b, double* z_o
 // z = C^+ b by the factor; *used = false when the factor cannot serve this
 // mesh or this right-hand side (the caller then runs CG)
 int chol_solve(tp_mesh* m, const tp_params* p, const double* b, int k, double* z_out, cudaStream_t st, int* iters,
-               bool* used, bool deferred) {
+               bool* used, PoissonMode mode) {
     *used = false;
     if (k < 1 || k > CH_KMAX) return fail(TP_ERR_INVALID_ARG, "cotan solve: k must be in 1..9");
     TP_TRY(laplacian_values(m, st));
@@ -1653,15 +1666,15 @@ int chol_solve(tp_mesh* m, const tp_params* p, const double* b, int k, double* z
     bool handed = false;
     int it = 0;
     switch (k) {
-        case 1: TP_TRY(chol_run<1>(m, p, b, z_out, st, &it, &handed, deferred)); break;
-        case 2: TP_TRY(chol_run<2>(m, p, b, z_out, st, &it, &handed, deferred)); break;
-        case 3: TP_TRY(chol_run<3>(m, p, b, z_out, st, &it, &handed, deferred)); break;
-        case 4: TP_TRY(chol_run<4>(m, p, b, z_out, st, &it, &handed, deferred)); break;
-        case 5: TP_TRY(chol_run<5>(m, p, b, z_out, st, &it, &handed, deferred)); break;
-        case 6: TP_TRY(chol_run<6>(m, p, b, z_out, st, &it, &handed, deferred)); break;
-        case 7: TP_TRY(chol_run<7>(m, p, b, z_out, st, &it, &handed, deferred)); break;
-        case 8: TP_TRY(chol_run<8>(m, p, b, z_out, st, &it, &handed, deferred)); break;
-        default: TP_TRY(chol_run<9>(m, p, b, z_out, st, &it, &handed, deferred)); break;
+        case 1: TP_TRY(chol_run<1>(m, p, b, z_out, st, &it, &handed, mode)); break;
+        case 2: TP_TRY(chol_run<2>(m, p, b, z_out, st, &it, &handed, mode)); break;
+        case 3: TP_TRY(chol_run<3>(m, p, b, z_out, st, &it, &handed, mode)); break;
+        case 4: TP_TRY(chol_run<4>(m, p, b, z_out, st, &it, &handed, mode)); break;
+        case 5: TP_TRY(chol_run<5>(m, p, b, z_out, st, &it, &handed, mode)); break;
+        case 6: TP_TRY(chol_run<6>(m, p, b, z_out, st, &it, &handed, mode)); break;
+        case 7: TP_TRY(chol_run<7>(m, p, b, z_out, st, &it, &handed, mode)); break;
+        case 8: TP_TRY(chol_run<8>(m, p, b, z_out, st, &it, &handed, mode)); break;
+        default: TP_TRY(chol_run<9>(m, p, b, z_out, st, &it, &handed, mode)); break;
     }
     if (iters) *iters = it;
     *used = !handed;

@@ -76,21 +76,21 @@ int differential_dev(tp_mesh* m, const tp_params* p, double* dE, double* E_host,
 }
 
 // z = C^+ L^{2-s} C^+ b (§5.2); b, z [nv][k] device
-// With strict = false (inside flexible GMRES) an inner CG solve that stops at
+// In the modes of flexible GMRES an inner CG solve that stops at
 // its iteration cap still returns its iterate: the outer method only needs
 // some fixed-quality approximation of the preconditioner.
 int precond_apply_dev(tp_mesh* m, const tp_params* p, const double* b, int k, double* z,
-                      cudaStream_t st, int* cg_iters, bool strict) {
+                      cudaStream_t st, int* cg_iters, PoissonMode mode) {
     const size_t n = (size_t)m->nv * k;
     TP_TRY(ensure(m->prec[0], sizeof(double) * n));
     TP_TRY(ensure(m->prec[1], sizeof(double) * n));
     int it1 = 0, it2 = 0;
     // with pins the pin rows are appended to both Laplacians (§7.2)
-    // inside flexible GMRES (strict = false) the factorised solves run
-    // deferred: no host read per solve; the step reads their flags once
     auto solve = [&](const double* rhs, double* out, int* it) {
-        return m->npins ? pinned_solve(m, p, rhs, k, out, st, it) : cg_solve(m, p, rhs, k, out, st, it, !strict);
+        return m->npins ? pinned_solve(m, p, rhs, k, out, st, it)
+                        : cg_solve(m, p, rhs, k, out, st, it, mode);
     };
+    const bool strict = mode == POISSON_STRICT;
     int s1 = solve(b, m->prec[0].as<double>(), &it1);
     if (s1 != TP_OK && (strict || s1 != TP_ERR_NOT_CONVERGED)) return s1;
     // (the second solve projects its right-hand side itself, or ignores its pinned rows)
@@ -254,6 +254,13 @@ static int fgmres_multi(tp_mesh* m, const tp_params* p, int ns, const double* co
     }
     auto Vj = [&](GmSys& q, int j) { return q.V + (size_t)j * n; };
     auto Zj = [&](GmSys& q, int j) { return q.Z + (size_t)j * n; };
+    // The fixed number of sweeps of the deferred solves suits meshes of ordinary triangles.
+    // On needles the FP32 factor gains less than a digit a sweep or stalls, which on large
+    // meshes CG had caught: there the first application's solves are looked at (one host
+    // wait), and where more than a hundredth of a right-hand side was left, it and all others
+    // of this call sweep on to cg_tol or hand over to CG.
+    const bool large = nv > CHOL_LARGE_NV;
+    PoissonMode mode = POISSON_DEFERRED;
     int total = 0;
     for (;;) {
         std::vector<int> act;
@@ -280,7 +287,16 @@ static int fgmres_multi(tp_mesh* m, const tp_params* p, int ns, const double* co
                 wout.push_back(S[i].w);
             }
             TP_TRY(pack(vin, nv, P0, st));
-            TP_TRY(precond_apply_dev(m, p, P0, 3 * na, P1, st, &ks->cg_iters, false));
+            TP_TRY(precond_apply_dev(m, p, P0, 3 * na, P1, st, &ks->cg_iters, mode));
+            if (total == 0 && large) {
+                int err = 0, poor = 0;
+                TP_TRY(chol_deferred_flags(m, st, &err, &poor, false));
+                if (err) return fail(TP_ERR_TIMEOUT, "precond_step: a wait of the factorised sweep gave up");
+                if (poor) {
+                    mode = POISSON_LOOSE;
+                    TP_TRY(precond_apply_dev(m, p, P0, 3 * na, P1, st, &ks->cg_iters, mode));
+                }
+            }
             TP_TRY(unpack(P1, nv, zout, st));
             TP_TRY(apply_A_unpacked(m, p, P1, na, P2, wout, st));
             ++total;
@@ -735,11 +751,11 @@ int precond_step_dev(tp_mesh* m, const tp_params* p, const tp_constraints* c, tp
     r.krylov_iters = ks.iters;
     r.cg_iters = ks.cg_iters;
     {
-        // the deferred Poisson solves of the Krylov loop: a wait that gave up
-        // is an error; solves that stopped short of cg_tol only made the
-        // (flexible) preconditioner less exact
-        int derr = 0, dunc = 0;
-        TP_TRY(chol_deferred_flags(m, st, &derr, &dunc, false));
+        // the deferred Poisson solves of the Krylov loop: a wait that gave up is an error;
+        // solves that stopped short of cg_tol only made the (flexible) preconditioner less
+        // exact
+        int derr = 0, poor = 0;
+        TP_TRY(chol_deferred_flags(m, st, &derr, &poor, false));
         if (derr) return fail(TP_ERR_TIMEOUT, "precond_step: a wait of the factorised sweep gave up");
         int tcerr = 0;
         if (p->tensor_cores) TP_TRY(apply_tc_error(m, &tcerr, st));

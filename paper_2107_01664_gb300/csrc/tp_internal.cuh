@@ -459,8 +459,13 @@ int bh_lists(tp_mesh* m, const tp_params* p, cudaStream_t st, BhLists* out, bool
 // -------- cg.cu ------------------------------------------------------------
 int laplacian_setup(tp_mesh* m);                        // CSR pattern (host, once)
 int laplacian_values(tp_mesh* m, cudaStream_t st);      // cotan values for current positions
+// how a Poisson solve ends: STRICT reaches cg_tol or fails; inside flexible GMRES, DEFERRED
+// runs a fixed number of sweeps with no host read (see chol_deferred_flags), and LOOSE
+// sweeps to cg_tol but takes a stalled iterate with a hundredth of the right-hand side left
+// (more: CG)
+enum PoissonMode { POISSON_STRICT, POISSON_DEFERRED, POISSON_LOOSE };
 int cg_solve(tp_mesh* m, const tp_params* p, const double* b_dev, int k, double* z_dev,
-             cudaStream_t st, int* iters, bool deferred = false);
+             cudaStream_t st, int* iters, PoissonMode mode = POISSON_STRICT);
 // y += G x (k columns), G the within-face term of the preconditioner's
 // L^{2-s} with weight p->prec_self_weight (nothing when the weight is 0)
 int self_term_add(tp_mesh* m, const tp_params* p, const double* x_dev, int k, double* y_dev,
@@ -469,11 +474,13 @@ int self_term_add(tp_mesh* m, const tp_params* p, const double* x_dev, int k, do
 // z = C^+ b through the sparse Cholesky factor; *used = false when the
 // factor cannot serve the mesh (panel too large) or refinement stalled
 int chol_solve(tp_mesh* m, const tp_params* p, const double* b_dev, int k, double* z_dev,
-               cudaStream_t st, int* iters, bool* used, bool deferred = false);
-// deferred solves (deferred = true: no host read per solve, the sweeps cg_tol
-// needs, flags accumulated on the device): read (unless reset) and clear the
-// accumulated wait error and unconverged-solve flags
-int chol_deferred_flags(tp_mesh* m, cudaStream_t st, int* err, int* unconverged, bool reset);
+               cudaStream_t st, int* iters, bool* used, PoissonMode mode = POISSON_STRICT);
+// deferred solves (flags accumulated on the device): read (unless reset) and clear the
+// accumulated wait error and whether a solve fell short of cg_tol with more than a
+// hundredth of a right-hand side left
+// more vertices than this: fewer digits a sweep of the deferred solves (see chol_run)
+constexpr int CHOL_LARGE_NV = 120000;
+int chol_deferred_flags(tp_mesh* m, cudaStream_t st, int* err, int* poor, bool reset);
 int chol_info(tp_mesh* m, tp_chol_info* out);
 // waits in one kernel on a word nothing sets: TP_ERR_TIMEOUT and *timed_out = 1
 // once the bounded wait gives up (current device)
@@ -533,7 +540,7 @@ int energy_value(tp_mesh* m, const tp_params* p, double* E_host, cudaStream_t st
 int differential_dev(tp_mesh* m, const tp_params* p, double* dE_dev, double* E_host,
                      cudaStream_t st, bool aux = false);
 int precond_apply_dev(tp_mesh* m, const tp_params* p, const double* b, int k, double* z,
-                      cudaStream_t st, int* cg_iters, bool strict = true);
+                      cudaStream_t st, int* cg_iters, PoissonMode mode = POISSON_STRICT);
 int precond_step_dev(tp_mesh* m, const tp_params* p, const tp_constraints* c, tp_step_report* rep,
                      cudaStream_t st);
 // total area (§7.1.3) and enclosed signed volume (§7.1.4) of the current positions (host)
