@@ -289,7 +289,7 @@ typedef struct tp_chol_info {
     int    levels;         /* tree height + 1 (sequential launches per substitution) */
     int    max_front;      /* largest front (own + structure rows) */
     double factor_floats;  /* stored factor entries (L11^-1 and L21 blocks) */
-    double update_floats;  /* update-matrix entries */
+    double update_floats;  /* update-matrix entries stored (0 if the solver does not serve the mesh) */
 } tp_chol_info;
 
 int cotan_factor_info(tp_mesh* m, tp_chol_info* out);

@@ -74,6 +74,7 @@ struct CholState {
     std::vector<size_t> lvl_factor_smem;  // bytes
     std::vector<int> lvl_tile;            // first entry of each level in `tiles`
     std::vector<double> lvl_factor_flops;
+    int64_t usize = 0;                    // floats of the update matrices (those in place share their child's)
     double solve_bytes = 0.0;             // factor bytes read by one forward + backward sweep
     Buf nodes, level_nodes, child_idx, rel, struct_pos, asm_dst, asm_src, perm, comp_ptr, comp_verts, comp_of;
     Buf parent, fdone, bdone, trace, tiles;
@@ -1294,7 +1295,7 @@ static int chol_setup(tp_mesh* m) {
     // update matrices: in place ones are the trailing part of the child's
     std::vector<int64_t> uoff(S.nnode);
     std::vector<int> ldu(S.nnode);
-    int64_t usize = 0;
+    int64_t& usize = c->usize;
     for (int J = 0; J < S.nnode; ++J) {   // postorder: children first
         if (flags[J] & CHN_INPLACE) {
             const int ch = S.child_idx[S.child_ptr[J]];
@@ -1735,7 +1736,7 @@ int chol_info(tp_mesh* m, tp_chol_info* out) {
     out->levels = c->H;
     out->max_front = S.max_t;
     out->factor_floats = (double)S.lsize;
-    out->update_floats = (double)S.usize;
+    out->update_floats = (double)c->usize;
     return TP_OK;
 }
 
