@@ -10,7 +10,7 @@
 // traversal needs no stack. The shape depends only on (nf, leaf_size) and
 // is built once per mesh; the Morton order and the node data (area a_I,
 // area-weighted barycenter X_I, bounding box of the faces' vertices, radius
-// r_I from X_I) are rebuilt bottom-up whenever the positions change. With
+// r_I from X_I) are rebuilt from the leaves up whenever the positions change. With
 // bvh_refit the face order of the last build is kept and only the node data
 // are recomputed: any face order gives a valid tree (the admissibility test
 // uses the actual boxes and radii), only its quality drifts.
@@ -50,8 +50,8 @@ struct NodeShape {  // fixed per mesh
 // host: implicit tree shape
 // ---------------------------------------------------------------------------
 
-static void shape_rec(std::vector<NodeShape>& out, std::vector<int>& depth, std::vector<int>& left,
-                      int id, int lo, int hi, int d, int leaf, int nf) {
+// (returns the depth of the subtree's deepest leaf)
+static int shape_rec(std::vector<NodeShape>& out, int id, int lo, int hi, int d, int leaf, int nf) {
     int n = hi - lo;
     NodeShape s;
     s.first = lo * leaf;
@@ -59,49 +59,26 @@ static void shape_rec(std::vector<NodeShape>& out, std::vector<int>& depth, std:
     s.skip = id + 2 * n - 1;
     s.leaf = n == 1;
     out[id] = s;
-    depth[id] = d;
-    if (n == 1) {
-        left[id] = -1;
-        return;
-    }
+    if (n == 1) return d;
     int nl = (n + 1) / 2;
-    left[id] = id + 1;
-    shape_rec(out, depth, left, id + 1, lo, lo + nl, d + 1, leaf, nf);
-    shape_rec(out, depth, left, id + 2 * nl, lo + nl, hi, d + 1, leaf, nf);
+    const int dl = shape_rec(out, id + 1, lo, lo + nl, d + 1, leaf, nf);
+    const int dr = shape_rec(out, id + 2 * nl, lo + nl, hi, d + 1, leaf, nf);
+    return std::max(dl, dr);
 }
 
 struct BvhHost {
     int leaf = 0, nleaf = 0, nnodes = 0, maxdepth = 0;
-    std::vector<int> level_off;  // nodes sorted by depth: offsets per depth
 };
 
-// device arrays in m->bvh_tmp: [shape int4 nnodes][right child int][level order int]
+// the nodes' shapes on the device, in m->bvh_tmp
 static int bvh_shape(tp_mesh* m, int leaf, BvhHost& h) {
     h.leaf = leaf;
     h.nleaf = (m->nf + leaf - 1) / leaf;
     h.nnodes = 2 * h.nleaf - 1;
     std::vector<NodeShape> sh(h.nnodes);
-    std::vector<int> depth(h.nnodes), left(h.nnodes);
-    shape_rec(sh, depth, left, 0, 0, h.nleaf, 0, leaf, m->nf);
-    h.maxdepth = *std::max_element(depth.begin(), depth.end());
-    std::vector<int> order(h.nnodes);
-    for (int i = 0; i < h.nnodes; ++i) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return depth[a] < depth[b]; });
-    h.level_off.assign(h.maxdepth + 2, 0);
-    for (int i = 0; i < h.nnodes; ++i) h.level_off[depth[i] + 1]++;
-    for (int d = 0; d <= h.maxdepth; ++d) h.level_off[d + 1] += h.level_off[d];
-    // right child = first node after the left subtree = escape index of the left child
-    std::vector<int> right(h.nnodes, -1);
-    for (int i = 0; i < h.nnodes; ++i)
-        if (!sh[i].leaf) right[i] = sh[i + 1].skip;
-    size_t bytes = sizeof(NodeShape) * h.nnodes + sizeof(int) * 2 * (size_t)h.nnodes;
-    TP_TRY(ensure(m->bvh_tmp, bytes));
-    char* base = m->bvh_tmp.as<char>();
-    TP_CUDA(cudaMemcpy(base, sh.data(), sizeof(NodeShape) * h.nnodes, cudaMemcpyHostToDevice));
-    TP_CUDA(cudaMemcpy(base + sizeof(NodeShape) * h.nnodes, right.data(), sizeof(int) * h.nnodes,
-                       cudaMemcpyHostToDevice));
-    TP_CUDA(cudaMemcpy(base + sizeof(NodeShape) * h.nnodes + sizeof(int) * h.nnodes, order.data(),
-                       sizeof(int) * h.nnodes, cudaMemcpyHostToDevice));
+    h.maxdepth = shape_rec(sh, 0, 0, h.nleaf, 0, leaf, m->nf);
+    TP_TRY(ensure(m->bvh_tmp, sizeof(NodeShape) * h.nnodes));
+    TP_CUDA(cudaMemcpy(m->bvh_tmp.ptr, sh.data(), sizeof(NodeShape) * h.nnodes, cudaMemcpyHostToDevice));
     return TP_OK;
 }
 
@@ -368,7 +345,6 @@ int bvh_build(tp_mesh* m, const tp_params* p, cudaStream_t st) {
         m->bvh_shape_leaf = h.leaf;
         m->bvh_maxdepth = h.maxdepth;
         m->bvh_nodes = h.nnodes;
-        m->bvh_level_off = h.level_off;
         m->bvh_valid = false;
         m->bvh_ordered = false;
     }
@@ -377,7 +353,6 @@ int bvh_build(tp_mesh* m, const tp_params* p, cudaStream_t st) {
     h.leaf = m->bvh_shape_leaf;
     h.nnodes = m->bvh_nodes;
     h.maxdepth = m->bvh_maxdepth;
-    h.level_off = m->bvh_level_off;
     const int nf = m->nf;
     m->bvh_nodes = h.nnodes;
     m->bvh_leaf = h.leaf;
@@ -406,8 +381,6 @@ int bvh_build(tp_mesh* m, const tp_params* p, cudaStream_t st) {
     d4* node64 = na.node64;
     float4* nodelo = na.nodelo;
     const NodeShape* shape = m->bvh_tmp.as<NodeShape>();
-    const int* right = (const int*)(shape + h.nnodes);
-    const int* order = right + h.nnodes;
 
     ProfScope ps(m, PK_BVH_BUILD, (double)nf, st);
     if (p->bvh_refit && m->bvh_ordered) {
@@ -458,10 +431,7 @@ int bvh_build(tp_mesh* m, const tp_params* p, cudaStream_t st) {
 int bvh_view(tp_mesh* m, const tp_params* p, cudaStream_t st, BvhView* v) {
     TP_TRY(bvh_build(m, p, st));
     const NodeArrays na = node_arrays(m);
-    const NodeShape* shape = m->bvh_tmp.as<NodeShape>();
-    const int* right = (const int*)(shape + m->bvh_nodes);
     v->nnodes = m->bvh_nodes;
-    v->maxdepth = m->bvh_maxdepth;
     v->node = na.node;
     v->nodelo = na.nodelo;
     v->sa = m->bvh_f32a.as<float4>();
@@ -469,9 +439,6 @@ int bvh_view(tp_mesh* m, const tp_params* p, cudaStream_t st, BvhView* v) {
     v->sl = m->bvh_f32c.as<float4>();
     v->perm = m->bvh_perm.as<int>();
     v->fbox = (const FaceBox*)(v->perm + m->nf);
-    v->right = right;
-    v->level_order = right + m->bvh_nodes;
-    v->level_off = m->bvh_level_off.data();
     return TP_OK;
 }
 
@@ -835,7 +802,7 @@ size_t bh_footprint_bytes(int nf, int leaf, double theta) {
     const size_t chunks = bhl_first_chunks(nf, theta);
     const size_t tree = F * (sizeof(int) + sizeof(FaceBox) + 3 * sizeof(float4)) + F * 8 + 65536 +
                         std::max(F * 16 + 49200, nn * (sizeof(d4) + 12)) + node_bytes((int)nn) +
-                        nn * (sizeof(NodeShape) + 8);
+                        nn * sizeof(NodeShape);
     const size_t lists = chunks * (BHL_CHUNK_BYTES + sizeof(int2) * BHL_CHUNK) + groups * 32 + 65536;
     return tree + lists + 16 * (10 * F + 12 * nn) + 44 * nn + F * 16;
 }
@@ -1744,8 +1711,7 @@ __global__ void k_node_push_terms(double* __restrict__ nacc, const d4* __restric
 
 // per sorted face i: walk root -> leaf of i summing the node terms, then
 // assemble the FP64 face adjoints (face order) from target and source sides
-__global__ void k_bh_diff_combine(const NodeShape* __restrict__ shape, const int* __restrict__ right, int nnodes,
-                                  int leaf, const int* __restrict__ perm, int nf, const double* __restrict__ tacc,
+__global__ void k_bh_diff_combine(int nnodes, int leaf, const int* __restrict__ perm, int nf, const double* __restrict__ tacc,
                                   const double* __restrict__ nacc, const double* __restrict__ facc,
                                   const d4* __restrict__ f64a, const d4* __restrict__ f64b, double p, int full,
                                   double* __restrict__ adj, double* __restrict__ erow) {
@@ -1849,9 +1815,7 @@ int diff_adjoints_bh(tp_mesh* m, const tp_params* p, double* adj, double* erow, 
         k_node_push_terms<<<(nn + 255) / 256, 256, 0, st>>>(nacc, node64, nn);
         TP_LAUNCH_CHECK();
     }
-    const NodeShape* shape = m->bvh_tmp.as<NodeShape>();
-    const int* right = (const int*)(shape + nn);
-    k_bh_diff_combine<<<(nf + 255) / 256, 256, 0, st>>>(shape, right, nn, m->bvh_leaf, perm, nf, tacc, nacc, facc,
+    k_bh_diff_combine<<<(nf + 255) / 256, 256, 0, st>>>(nn, m->bvh_leaf, perm, nf, tacc, nacc, facc,
                                                         m->f64a.as<d4>(), m->f64b.as<d4>(), p->p, full ? 1 : 0,
                                                         adj, erow);
     TP_LAUNCH_CHECK();

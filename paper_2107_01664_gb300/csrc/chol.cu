@@ -8,7 +8,7 @@
 //   factor (two launches per tree level): k_chol_panel, one block per supernode
 //   J, assembles the panel (t x nJ, shared memory) from the entries of C in J's
 //   columns and the children's update matrices, factors its diagonal block
-//   (right-looking, column by column) with L11^-1 formed along the way, and
+//   (right-looking, in blocks of eight columns) with L11^-1 formed along the way, and
 //   stores L11^-1 and L21; k_chol_update, one block per 64 x 64 tile, forms
 //   U_J = (children's share of struct x struct) - L21 L21^T (global memory).
 //
@@ -70,7 +70,7 @@ struct CholState {
     bool ok = false;
     std::string why;
     int H = 0;                            // number of levels
-    std::vector<int> lvl_max_t, lvl_max_n, lvl_max_m;
+    std::vector<int> lvl_max_t;           // rows of the level's largest front
     std::vector<size_t> lvl_factor_smem;  // bytes
     std::vector<int> lvl_tile;            // first entry of each level in `tiles`
     std::vector<double> lvl_factor_flops;
@@ -80,7 +80,7 @@ struct CholState {
     Buf parent, fdone, bdone, trace, tiles;
     // dynamic shared memory of the sweep kernel by column count: the largest of all
     // nodes, and of the leading tree levels that leave room for three blocks per SM
-    // (small_n nodes, small_lvls levels)
+    // (small_n nodes)
     size_t solve_smem[CH_KMAX + 1] = {}, small_smem[CH_KMAX + 1] = {};
     int small_n[CH_KMAX + 1] = {};
     bool wide = false;         // a front has more than 256 rows, or CHN_DIRECT
@@ -90,15 +90,15 @@ struct CholState {
     // refinement sweeps captured as CUDA graphs, one per column count, keyed
     // by the buffers and scalars baked into their launches
     // deferred solves (inside flexible GMRES): the pivot check of the current
-    // factor is read once, and the sweeps' wait errors and unconverged
-    // columns accumulate in dflags [2] for the caller to read once per step
+    // factor is read once, and the sweeps' wait errors and poor columns accumulate in
+    // dflags [2] for the caller to read (chol_deferred_flags)
     bool pivot_known = false, pivot_ok = false;
     Buf dflags;
     struct SweepGraph {
         cudaGraphExec_t exec = nullptr;
         const void* key[4] = {};
         double tol2 = 0.0;
-        int cap = 0, rgrid = 0, kernels = 0;
+        int cap = 0, kernels = 0;
     } graph[CH_KMAX + 1];
     cudaStream_t capture = nullptr;
 };
@@ -1233,8 +1233,6 @@ static int chol_setup(tp_mesh* m) {
     c->ncomp = S.ncomp;
     c->H = (int)S.level_ptr.size() - 1;
     c->lvl_max_t.assign(c->H, 0);
-    c->lvl_max_n.assign(c->H, 0);
-    c->lvl_max_m.assign(c->H, 0);
     c->lvl_factor_smem.assign(c->H, 0);
     c->lvl_factor_flops.assign(c->H, 0.0);
     // bytes of a solve step on K columns: the factor block (rounded to 16 bytes),
@@ -1259,8 +1257,6 @@ static int chol_setup(tp_mesh* m) {
             const int J = S.level_nodes[i];
             const double n = S.nJ[J], mm = S.mJ[J];
             c->lvl_max_t[h] = std::max(c->lvl_max_t[h], S.nJ[J] + S.mJ[J]);
-            c->lvl_max_n[h] = std::max(c->lvl_max_n[h], S.nJ[J]);
-            c->lvl_max_m[h] = std::max(c->lvl_max_m[h], S.mJ[J]);
             int child = 0;   // rows of the largest child
             for (int ci = S.child_ptr[J]; ci < S.child_ptr[J + 1]; ++ci) child = std::max(child, S.mJ[S.child_idx[ci]]);
             const size_t sm = chf_smem((size_t)S.nJ[J] + S.mJ[J], S.nJ[J], child);
@@ -1438,8 +1434,7 @@ static int comp_project(tp_mesh* m, const double* src, double* dst, int k, cudaS
 // `nsweep` refinement sweeps on stream st (recorded into a graph by the
 // caller); *nk counts the kernels
 template <int K>
-static int chol_sweep_kernels(tp_mesh* m, int nsweep, int rgrid, double* partr, double tol2, int cap,
-                              cudaStream_t st, int* nk) {
+static int chol_sweep_kernels(tp_mesh* m, int nsweep, double* partr, double tol2, int cap, cudaStream_t st, int* nk) {
     CholState* c = m->chol;
     const CholSymbolic& S = c->S;
     SweepArgs A;
@@ -1472,7 +1467,6 @@ static int chol_sweep_kernels(tp_mesh* m, int nsweep, int rgrid, double* partr, 
     A.nv = m->nv;
     A.nn = S.nnode;
     A.cap = cap;
-    (void)rgrid;
     const int nn = S.nnode, sms = sm_count(), small = c->small_n[K];
     // One launch a sweep, with the shared memory of its largest step. Where that
     // leaves one or two blocks per SM to thousands of small steps (163,842 vertices:
@@ -1508,11 +1502,11 @@ constexpr int CH_SWEEPS_PER_GRAPH = 2;   // FP32 factor: about three digits per 
 // the graph of CH_SWEEPS_PER_GRAPH sweeps for K columns, captured on a
 // private stream (re-captured when a buffer it uses has moved)
 template <int K>
-static int sweep_graph(tp_mesh* m, int rgrid, double* partr, double tol2, int cap, CholState::SweepGraph** out) {
+static int sweep_graph(tp_mesh* m, double* partr, double tol2, int cap, CholState::SweepGraph** out) {
     CholState* c = m->chol;
     CholState::SweepGraph& g = c->graph[K];
     const void* key[4] = {c->x.ptr, c->r.ptr, c->bp.ptr, partr};
-    bool same = g.exec && g.tol2 == tol2 && g.cap == cap && g.rgrid == rgrid;
+    bool same = g.exec && g.tol2 == tol2 && g.cap == cap;
     for (int i = 0; i < 4 && same; ++i) same = g.key[i] == key[i];
     if (!same) {
         if (g.exec) cudaGraphExecDestroy(g.exec);
@@ -1520,7 +1514,7 @@ static int sweep_graph(tp_mesh* m, int rgrid, double* partr, double tol2, int ca
         if (!c->capture) TP_CUDA(cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking));
         TP_CUDA(cudaStreamBeginCapture(c->capture, cudaStreamCaptureModeThreadLocal));
         int nk = 0;
-        int s = chol_sweep_kernels<K>(m, CH_SWEEPS_PER_GRAPH, rgrid, partr, tol2, cap, c->capture, &nk);
+        int s = chol_sweep_kernels<K>(m, CH_SWEEPS_PER_GRAPH, partr, tol2, cap, c->capture, &nk);
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(c->capture, &graph);
         if (s != TP_OK) {
@@ -1536,7 +1530,6 @@ static int sweep_graph(tp_mesh* m, int rgrid, double* partr, double tol2, int ca
         for (int i = 0; i < 4; ++i) g.key[i] = key[i];
         g.tol2 = tol2;
         g.cap = cap;
-        g.rgrid = rgrid;
         g.kernels = nk;
     }
     *out = &g;
@@ -1589,7 +1582,7 @@ static int chol_run(tp_mesh* m, const tp_params* p, const double* b, double* z_o
     const double tol2 = p->cg_tol * p->cg_tol;
     const int cap = std::max(1, std::min(p->cg_max, 40));
     CholState::SweepGraph* g = nullptr;
-    TP_TRY(sweep_graph<K>(m, rgrid, partr, tol2, cap, &g));
+    TP_TRY(sweep_graph<K>(m, partr, tol2, cap, &g));
     if (deferred) {
         // no host read: a fixed number of sweeps for cg_tol, then the flags, which
         // the caller reads. Measured digits of |r|/|b| (9 columns, random b): at
@@ -1619,7 +1612,7 @@ static int chol_run(tp_mesh* m, const tp_params* p, const double* b, double* z_o
             // the odd sweep, launched directly
             ProfScope ps(m, PK_CHOL_SOLVE, c->solve_bytes, st);
             int nk = 0;
-            TP_TRY(chol_sweep_kernels<K>(m, sweeps % CH_SWEEPS_PER_GRAPH, rgrid, partr, tol2, cap, st, &nk));
+            TP_TRY(chol_sweep_kernels<K>(m, sweeps % CH_SWEEPS_PER_GRAPH, partr, tol2, cap, st, &nk));
             count_launches(nk);
         }
         if (iters) *iters = sweeps;

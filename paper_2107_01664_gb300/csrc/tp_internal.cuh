@@ -212,7 +212,7 @@ struct BhLists {
 
 // read-only view of a built tree for kernels outside bvh.cu
 struct BvhView {
-    int nnodes = 0, maxdepth = 0;
+    int nnodes = 0;
     const BvhNode* node = nullptr;
     const float4* nodelo = nullptr;      // low parts of the node barycenters
     const float4* sa = nullptr;          // sorted faces: X - c, a
@@ -220,9 +220,6 @@ struct BvhView {
     const float4* sl = nullptr;          // sorted faces: low parts of X - c
     const FaceBox* fbox = nullptr;
     const int* perm = nullptr;           // sorted position -> face
-    const int* right = nullptr;          // right child of an inner node
-    const int* level_order = nullptr;    // nodes grouped by depth
-    const int* level_off = nullptr;      // host: offsets of the depths in level_order
 };
 
 // packed float2 arithmetic (two IEEE lanes per instruction)
@@ -333,7 +330,6 @@ struct tp_mesh {
     // Barnes-Hut tree (rebuilt per positions on demand)
     int bvh_nodes = 0, bvh_leaf = 0;
     int bvh_shape_leaf = 0, bvh_maxdepth = 0;
-    std::vector<int> bvh_level_off;
     bool bvh_valid = false;
     bool bvh_ordered = false;     // perm holds a face order for the current leaf size (refit keeps it)
     tp::Buf bvh_node, bvh_perm, bvh_keys, bvh_tmp, bvh_sortws;
