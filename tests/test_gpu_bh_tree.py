@@ -70,3 +70,40 @@ def test_lists_longer_than_the_first_pool(lib, noise, theta, leaf):
     assert E[0] == E[1] == E[2]
     assert np.array_equal(y[0], y[1]) and np.array_equal(y[0], y[2])
     assert abs(E[0] / rows.sum() - 1) <= TOL
+
+
+def test_lists_without_room_for_the_pool(lib):
+    # an allocator that refuses the pool (43 MB here; nothing else is above 16 MB): two
+    # traversals give the same lists, hence E and the apply bit by bit
+    import ctypes
+
+    import torch
+    from synth import gaussian_noise, torus
+    V, F = torus(200, 50, 1.0, 0.3)
+    V = gaussian_noise(V, 0.002, 1)
+    u = vertex_vectors(len(V), 3, 8)
+    p = lib.params(theta=0.25)
+    with lib.Mesh(V, F) as m:
+        E, y = lib.tp_energy(m, p), lib.fractional_apply(m, "A", u, p)
+    refused = []
+
+    @lib._ALLOC_FN
+    def alloc(nbytes, device, user):
+        if nbytes > 32 << 20:
+            refused.append(nbytes)
+            return None
+        return int(torch.cuda.caching_allocator_alloc(int(nbytes), device, torch.cuda.current_stream(device)))
+
+    @lib._FREE_FN
+    def free(ptr, nbytes, device, user):
+        torch.cuda.caching_allocator_delete(int(ptr))
+
+    with lib.Context(0) as ctx:
+        a = lib.tp_allocator(alloc, free, None)
+        lib._check(lib.lib().tp_ctx_set_allocator(ctx.handle, ctypes.byref(a)))
+        with lib.Mesh(V, F, ctx=ctx) as m:
+            for _ in range(2):
+                assert lib.tp_energy(m, p) == E
+                assert np.array_equal(lib.fractional_apply(m, "A", u, p), y)
+                m.set_positions(V)
+    assert len(refused) == 2
